@@ -101,6 +101,7 @@ static void free_device(Factors &F) {
                     F.d_pi_work, F.d_dense_loop};
     for (void *p : ptrs)
         if (p && p != F.d_arena) cudaFree(p);
+    slab_free(F);
     // the arena came from the pool: returned in stream order (every call on
     // this object has synchronised with its stream before returning)
     if (F.d_arena) cudaFreeAsync(F.d_arena, 0);

@@ -3,7 +3,9 @@
 // transition tensor, mode products as in Kolda and Bader), followed by
 // Eq. 1's + R, x gamma and max over actions, and the residual.
 //
-// SIMT path: one tiled mode-product kernel per (action, rank, mode). The
+// SIMT path: the fused mode-product chains of dense_slab.cuh. Models that have
+// no plan there (a mode too large for one block's tile, or no memory for the
+// intermediates) run one tiled mode-product kernel per (action, rank, mode). The
 // mode-d product of X (viewed as L x N_d x Rt, Rt = prod of the later mode
 // sizes) with U is the batched matrix product Y[l, i, r] = sum_j U[i, j]
 // X[l, j, r]; columns c = (l, r) are tiled 64 at a time, rows i 64 at a
@@ -19,11 +21,10 @@
 #include <type_traits>
 #include <vector>
 
+#include "dense_slab.cuh"
 #include "internal.h"
 
 namespace cpmdp {
-
-enum DenseMode : int { DM_VI = 0, DM_EVAL = 1, DM_IMPROVE = 2, DM_GREEDY = 3, DM_STORE_E = 4 };
 
 struct Epilogue {
     int enabled;           // 0: plain store of Y (intermediate mode)
@@ -211,12 +212,16 @@ cpmdp_status dense_prepare(Factors &F) {
     // action: 5 x |S| doubles; argmax |S| bytes
     F.dense_work_bytes = 5 * S * sizeof(double) + S + 256;
     CPMDP_CUDA(cudaMalloc(&F.d_dense_work, F.dense_work_bytes));
-    return CPMDP_OK;
+    return slab_prepare(F);
 }
 
 template <typename T>
 static cpmdp_status dense_sweep(const Factors &F, const T *Vin, T *Vout, uint8_t *pi, int mode,
                                 double margin, unsigned long long *res, unsigned *chg, cudaStream_t st) {
+    if (slab_plan(F, sizeof(T))) {
+        CPMDP_CUDA(slab_sweep<T>(F, Vin, Vout, pi, mode, (T)margin, res, chg, st));
+        return CPMDP_OK;
+    }
     const size_t S = (size_t)F.nstates;
     T *work = (T *)F.d_dense_work;
     T *buf0 = work, *buf1 = work + S, *E = work + 2 * S, *best = work + 3 * S, *qold = work + 4 * S;

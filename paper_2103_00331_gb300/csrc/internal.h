@@ -43,6 +43,8 @@ struct Ctrl {
     unsigned long long bad_cell;   // factor build: 1 + index of a cell code other than 0, 1, 2 (0: none)
 };
 
+struct DenseSlab;
+
 struct Factors {
     int device = -1;
     int kind = CPMDP_GRIDWORLD;
@@ -103,6 +105,7 @@ struct Factors {
     void *d_dense_work = nullptr;      // dense chain intermediates
     size_t dense_work_bytes = 0;
     double *d_Vd = nullptr;            // dense FP64 certify: the float values as doubles
+    DenseSlab *slab = nullptr;  // fused mode-product chains: plans, factors, workspace (dense_slab.cuh)
     // dense tensor-core path (64^4), allocated on first BF16X3 use
     float *d_RB = nullptr;             // rewards in the pass-B layout
     void *d_T = nullptr;               // per-chain intermediates (bf16 hi/lo pairs)
@@ -188,6 +191,7 @@ cpmdp_status dense_backup(const Factors &F, cpmdp_precision prec, const void *Vi
 cpmdp_status dense_solve(const Factors &F, cpmdp_precision prec, bool policy_iteration, void *V,
                          uint8_t *pi, const SolveOpts &o, Ctrl *host_ctrl, cudaStream_t st);
 cpmdp_status dense_prepare(Factors &F);
+void slab_free(Factors &F);
 // dense_tc.cu
 bool dense_tc_supported(const Factors &F);
 cpmdp_status dense_tc_backup(const Factors &F, const float *Vin, float *Vout, uint8_t *pi, double *res,
