@@ -15,7 +15,9 @@
 //                    forward (s = +1, B_t[co, ci] = W[t, co, ci]) and data
 //                    gradient (s = -1, B_t[ci, co] = W[t, co, ci], times the
 //                    ReLU mask of the layer input)
-//   conv_dw_kernel   dW[t, co, ci] = sum_v dy[v, co] x[v + d off(t), ci] (SIMT)
+//   conv_dw_tma_kernel  dW[t, co, ci] = sum_v dy[v, co] x[v + d off(t), ci], the voxels as the
+//                    contraction of the same tensor cores (conv_dw_kernel: the SIMT
+//                    form, for operands that no tensor copy can address)
 //   plus features / targets / upsampling from a packed batch, the coarse
 //   value iteration, the cell-level and full-grid loss gradients, Adam and
 //   the FP32 -> BF16 weight casts.
@@ -117,7 +119,8 @@ __device__ __forceinline__ bool tm_wait(uint64_t *bar, uint32_t phase, volatile 
     return true;
 }
 
-__device__ __forceinline__ void tile_origin(const ConvGeo &g, int tile, int &nn, int &x0, int &y0, int &z0) {
+template <typename Geo>
+__device__ __forceinline__ void tile_origin(const Geo &g, int tile, int &nn, int &x0, int &y0, int &z0) {
     int r = tile;
     const int ix = r % g.tx; r /= g.tx;
     const int iy = r % g.ty; r /= g.ty;
@@ -334,6 +337,174 @@ __global__ void __launch_bounds__(kTmThreads, 1) conv_tma_kernel(const __grid_co
     if (warp == 5) tc::tmem_dealloc(tmem, kTmCols);
 }
 
+// ---------------------------------------------------------------------------
+// weight gradient on the tensor cores
+//
+// dW[t] is a 64 x 64 product contracted over all voxels, for 27 taps that read
+// the same dy and shifted copies of the same x. A CTA takes one (oz, ox) and
+// every splits-th tile of 128 voxels; the tile's dy and its shifted x arrive
+// by tensor copy (tall mode: one box of by + 2 d rows of y serves the three oy
+// taps; otherwise three boxes). Channels-last voxel rows are MN-major operands
+// as they lie, so nothing is transposed: A stacks two taps' 64 input channels
+// (two 64-wide MN atoms, the leading byte offset being the distance between
+// the taps' rows: oy = -1 and 0, then 0 again and 1), B is dy, K = 128 voxels.
+// The tensor cores truncate when they add to an accumulator, so a long chain
+// of them drifts (1.7e-6 off at 131,072 voxels when each CTA kept its sums in
+// TMEM to the end, 3.0e-7 on the FP32 pipe): each tile's sums (8 steps) are
+// drained and added up in registers, round to nearest, while the next tile
+// runs in the other TMEM buffer. At the end the CTA adds its sums to dW with
+// coalesced reductions.
+// A voxel of a tile beyond the grid has dy = 0 from the copy: it adds 0 x.
+// One layer at 32 x 16^3 voxels: 1,660 us on the FP32 pipe (conv_dw_kernel),
+// 68 us here (error against FP64 3.0e-7 and 1.8e-7); the x and dy copies run
+// at 4.9 TB/s from L2. One CTA for all nine taps of an oz with its sums kept
+// in TMEM took 38 us, at the error above.
+constexpr uint32_t kDwIdesc = tc::kIdescM128N64AMN | (1u << 16);   // A and B MN-major
+constexpr int kDwMaxStages = 6;
+
+struct DwGeo {
+    int n, z, y, x;
+    int bx, by, bz, tx, ty, tz, tiles, splits;
+    int tall, dil;
+    int xbytes, bstep;         // bytes of a tile's x boxes, between the rows of two oy
+    int stage_bytes, stages;
+};
+
+struct DwShared {
+    uint64_t full[kDwMaxStages], empty[kDwMaxStages], accf[2], acce[2];
+    uint32_t tslot;
+    int abort;
+};
+
+__global__ void __launch_bounds__(kTmThreads, 1) conv_dw_tma_kernel(const __grid_constant__ CUtensorMap tmx,
+                                                                    const __grid_constant__ CUtensorMap tmd,
+                                                                    float *__restrict__ dw, DwGeo g) {
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *sm = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    DwShared &S = *reinterpret_cast<DwShared *>(sm + (size_t)g.stages * g.stage_bytes);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int split = blockIdx.x / 9, oz = (int)(blockIdx.x % 9) / 3 - 1, ox = (int)(blockIdx.x % 3) - 1;
+    if (tid == 0) {
+        for (int i = 0; i < g.stages; i++) {
+            tc::mbar_init(&S.full[i], 1);
+            tc::mbar_init(&S.empty[i], 1);
+        }
+        for (int i = 0; i < 2; i++) {
+            tc::mbar_init(&S.accf[i], 1);
+            tc::mbar_init(&S.acce[i], 128);
+        }
+        S.abort = 0;
+    }
+    if (warp == 5) tc::tmem_alloc(&S.tslot, 256);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    tc::fence_proxy_async();
+    tc::fence_before();
+    __syncthreads();
+    tc::fence_after();
+    const uint32_t tmem = S.tslot;
+    volatile int *abort = &S.abort;
+    const int d = g.dil;
+
+    if (warp == 4) {
+        if (lane == 0) {
+            int last[kDwMaxStages];
+            for (int i = 0; i < kDwMaxStages; i++) last[i] = -1;
+            uint32_t count = 0;
+            for (int tile = split; tile < g.tiles; tile += g.splits, count++) {
+                const int st = (int)(count % (uint32_t)g.stages);
+                const uint32_t ph = (count / (uint32_t)g.stages) & 1;
+                if (count >= (uint32_t)g.stages && !tm_wait(&S.empty[st], ph ^ 1u, abort)) break;
+                int nn, x0, y0, z0;
+                tile_origin(g, tile, nn, x0, y0, z0);
+                const uint32_t dst = tc::smem_u32(sm + (size_t)st * g.stage_bytes);
+                const int xs = x0 + d * ox, zs = z0 + d * oz;
+                tc::mbar_expect_tx(&S.full[st], (uint32_t)g.xbytes + 16384u);
+                if (g.tall) {
+                    tc::tma_load_5d(dst, &tmx, 0, xs, y0 - d, zs, nn, &S.full[st]);
+                } else {
+                    for (int oy = 0; oy < 3; oy++)
+                        tc::tma_load_5d(dst + (uint32_t)(oy * g.bstep), &tmx, 0, xs, y0 + d * (oy - 1), zs, nn,
+                                        &S.full[st]);
+                }
+                tc::tma_load_5d(dst + (uint32_t)g.xbytes, &tmd, 0, x0, y0, z0, nn, &S.full[st]);
+                last[st] = (int)ph;
+            }
+            // every copy this thread issued lands before the CTA's shared memory goes
+            for (int i = 0; i < g.stages; i++)
+                if (last[i] >= 0) tc::mbar_wait(&S.full[i], (uint32_t)last[i], kCvWaitCycles);
+        }
+    } else if (warp == 5) {
+        if (lane == 0) {
+            uint32_t count = 0;
+            uint64_t *lastbar = nullptr;
+            uint32_t lastph = 0;
+            for (int tile = split; tile < g.tiles; tile += g.splits, count++) {
+                const int st = (int)(count % (uint32_t)g.stages), buf = count & 1;
+                if (count >= 2 && !tm_wait(&S.acce[buf], ((count >> 1) - 1) & 1, abort)) break;
+                if (!tm_wait(&S.full[st], (count / (uint32_t)g.stages) & 1, abort)) break;
+                tc::fence_after();
+                const uint32_t a0 = tc::smem_u32(sm + (size_t)st * g.stage_bytes), b0 = a0 + (uint32_t)g.xbytes;
+#pragma unroll
+                for (int i = 0; i < 2; i++)
+#pragma unroll
+                    for (int ks = 0; ks < 8; ks++)
+                        tc::mma(tmem + 128u * buf + 64u * i, tc::sdesc_mn(a0 + (uint32_t)(i * g.bstep) + ks * 2048u, (uint32_t)g.bstep),
+                                tc::sdesc_mn(b0 + ks * 2048u, 8192u), kDwIdesc, ks > 0 ? 1u : 0u);
+                tc::commit(&S.empty[st]);
+                tc::commit(&S.accf[buf]);
+                lastbar = &S.accf[buf];
+                lastph = (count >> 1) & 1;
+            }
+            // the MMAs complete in order: the last commit covers them all
+            if (lastbar) tc::mbar_wait(lastbar, lastph, kCvWaitCycles);
+        }
+    } else {
+        const int half = tid >> 6, ci = tid & 63;   // rows of A: 64 of oy = -1 (i = 1: 0), 64 of oy = 0 (1)
+        const uint32_t t0 = tmem + ((uint32_t)(32 * warp) << 16);
+        float acc[2][kC];
+#pragma unroll
+        for (int i = 0; i < 2; i++)
+#pragma unroll
+            for (int c = 0; c < kC; c++) acc[i][c] = 0.f;
+        bool ok = true;
+        uint32_t count = 0;
+        for (int tile = split; tile < g.tiles; tile += g.splits, count++) {
+            const int buf = count & 1;
+            ok = __all_sync(0xFFFFFFFFu, tm_wait(&S.accf[buf], (count >> 1) & 1, abort));
+            if (!ok) break;
+            tc::fence_after();
+#pragma unroll
+            for (int i = 0; i < 2; i++) {
+                if (i == 1 && half == 0) continue;   // oy = 0 again (whole warps)
+#pragma unroll
+                for (int h = 0; h < 2; h++) {
+                    float v[32];
+                    tc::tmem_ld32(t0 + 128u * buf + 64u * i + 32u * h, v);
+#pragma unroll
+                    for (int c = 0; c < 32; c++) acc[i][32 * h + c] += v[c];
+                }
+            }
+            tc::fence_before();
+            tc::mbar_arrive(&S.acce[buf]);
+        }
+        if (ok) {
+#pragma unroll
+            for (int i = 0; i < 2; i++) {
+                if (i == 1 && half == 0) continue;
+                float *o = dw + (size_t)((oz + 1) * 9 + (i + half) * 3 + ox + 1) * kC * kC + ci;
+#pragma unroll
+                for (int co = 0; co < kC; co++) atomicAdd(o + co * kC, acc[i][co]);
+            }
+        }
+    }
+    tc::fence_before();
+    __syncthreads();
+    tc::fence_after();
+    if (tid == 0 && S.abort) atomicExch(&g_conv_err, 1);
+    if (warp == 5) tc::tmem_dealloc(tmem, 256);
+}
+
+// The same on the FP32 pipe, for operands that are not 16-byte aligned:
 // dW[t, co, ci] += sum over a chunk of voxels of dy[v, co] x[v + d off(t), ci]
 __global__ void __launch_bounds__(256) conv_dw_kernel(const __nv_bfloat16 *__restrict__ x,
                                                       const __nv_bfloat16 *__restrict__ dy, float *__restrict__ dw,
@@ -390,7 +561,44 @@ __global__ void __launch_bounds__(256) conv_dw_kernel(const __nv_bfloat16 *__res
             atomicAdd(&dw[(size_t)t * kC * kC + (ty + 16 * i) * kC + tx + 16 * j], acc[i][j]);
 }
 
-// db[c] += sum_v dy[v, c]
+// db[c] += sum_v dy[v, c], 16 bytes (8 channels) a load: 8 lanes a voxel, 32
+// voxels a block at a time. Bound by the read of dy; one 2-byte load a thread
+// (conv_db_kernel) took 37 us for 131,072 voxels.
+__global__ void __launch_bounds__(256) conv_db_vec_kernel(const uint4 *__restrict__ dy, float *__restrict__ db, int nvox) {
+    __shared__ float sh[8][kC];
+    const int q = threadIdx.x & 7, warp = threadIdx.x >> 5;
+    float s[8];
+#pragma unroll
+    for (int k = 0; k < 8; k++) s[k] = 0.f;
+#pragma unroll 4
+    for (int v = blockIdx.x * 32 + (threadIdx.x >> 3); v < nvox; v += gridDim.x * 32) {
+        const uint4 m = dy[(size_t)v * 8 + q];
+        const uint32_t w[4] = {m.x, m.y, m.z, m.w};
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            s[2 * k] += __uint_as_float(w[k] << 16);
+            s[2 * k + 1] += __uint_as_float(w[k] & 0xFFFF0000u);
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < 8; k++) {
+        s[k] += __shfl_xor_sync(0xFFFFFFFFu, s[k], 8);
+        s[k] += __shfl_xor_sync(0xFFFFFFFFu, s[k], 16);
+    }
+    if ((threadIdx.x & 31) < 8) {
+#pragma unroll
+        for (int k = 0; k < 8; k++) sh[warp][8 * q + k] = s[k];
+    }
+    __syncthreads();
+    if (threadIdx.x < kC) {
+        float t = 0.f;
+#pragma unroll
+        for (int w = 0; w < 8; w++) t += sh[w][threadIdx.x];
+        atomicAdd(&db[threadIdx.x], t);
+    }
+}
+
+// The same for a dy that is not 16-byte aligned.
 __global__ void conv_db_kernel(const __nv_bfloat16 *__restrict__ dy, float *__restrict__ db, int nvox) {
     const int c = threadIdx.x & 63, lane_group = threadIdx.x >> 6;   // 4 groups of 64 threads
     float s = 0.f;
@@ -904,11 +1112,9 @@ static int pow2_at_least(int v) {
     return p;
 }
 
-// Tile shape, input ring and tensor map of one convolution launch.
-static cudaError_t launch_conv(const __nv_bfloat16 *x, const uint8_t *wimg, const float *bias,
-                               const __nv_bfloat16 *mask_act, __nv_bfloat16 *y, float *y0, Dims dm, int dil, int sign,
-                               int relu, cudaStream_t st) {
-    ConvGeo g;
+// Tiles of 128 voxels: a box of bx x by x bz.
+template <typename Geo>
+static bool tile_shape(const Dims &dm, int dil, Geo &g) {
     g.n = dm.n; g.z = dm.z; g.y = dm.y; g.x = dm.x;
     g.bx = std::min(16, std::max(8, pow2_at_least(dm.x)));
     g.by = std::min(128 / g.bx, pow2_at_least(dm.y));
@@ -917,35 +1123,49 @@ static cudaError_t launch_conv(const __nv_bfloat16 *x, const uint8_t *wimg, cons
     g.ty = (dm.y + g.by - 1) / g.by;
     g.tz = (dm.z + g.bz - 1) / g.bz;
     const long long tiles = (long long)g.tx * g.ty * g.tz * dm.n;
-    if (tiles > (1LL << 30)) return cudaErrorInvalidValue;
+    if (tiles > (1LL << 30)) return false;
     g.tiles = (int)tiles;
+    g.tall = g.bz == 1 && g.bx % 8 == 0 && g.by + 2LL * dil <= 256 && (g.by + 2LL * dil) * g.bx * 128 <= kTmAMax;
+    g.dil = dil;
+    return true;
+}
+
+// Tensor map of a channels-last activation, boxes of 64 channels x bx x rows x bz.
+static cudaError_t act_map(const __nv_bfloat16 *x, const Dims &dm, int bx, int rows, int bz, CUtensorMap *map) {
+    PFN_cuTensorMapEncodeTiled_v12000 enc = encode_tiled();
+    if (!enc) return cudaErrorNotSupported;
+    const cuuint64_t gdim[5] = {(cuuint64_t)kC, (cuuint64_t)dm.x, (cuuint64_t)dm.y, (cuuint64_t)dm.z, (cuuint64_t)dm.n};
+    const cuuint64_t gstride[4] = {(cuuint64_t)kC * 2, (cuuint64_t)kC * 2 * dm.x, (cuuint64_t)kC * 2 * dm.x * dm.y,
+                                   (cuuint64_t)kC * 2 * dm.x * dm.y * dm.z};
+    const cuuint32_t box[5] = {(cuuint32_t)kC, (cuuint32_t)bx, (cuuint32_t)rows, (cuuint32_t)bz, 1u};
+    const cuuint32_t estride[5] = {1u, 1u, 1u, 1u, 1u};
+    if (enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<__nv_bfloat16 *>(x), gdim, gstride, box, estride,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return cudaErrorInvalidValue;
+    return cudaSuccess;
+}
+
+// Tile shape, input ring and tensor map of one convolution launch.
+static cudaError_t launch_conv(const __nv_bfloat16 *x, const uint8_t *wimg, const float *bias,
+                               const __nv_bfloat16 *mask_act, __nv_bfloat16 *y, float *y0, Dims dm, int dil, int sign,
+                               int relu, cudaStream_t st) {
+    ConvGeo g;
+    if (!tile_shape(dm, dil, g)) return cudaErrorInvalidValue;
     const int tall_rows = (g.by + 2 * dil) * g.bx;
-    g.tall = g.bz == 1 && g.bx % 8 == 0 && g.by + 2 * dil <= 256 && tall_rows * 128 <= kTmAMax;
     g.stage_bytes = g.tall ? ((tall_rows * 128 + 1023) & ~1023) : kTmAMax;
     g.stages = std::min(kTmMaxStages,
                         (kTmSmemMax - 1024 - kTmBStages * kTmBStage - (int)sizeof(TmShared)) / g.stage_bytes);
-    g.dil = dil;
     g.sign = sign;
     g.relu = relu;
     const size_t smem = 1024 + (size_t)kTmBStages * kTmBStage + (size_t)g.stages * g.stage_bytes + sizeof(TmShared);
 
-    PFN_cuTensorMapEncodeTiled_v12000 enc = encode_tiled();
-    if (!enc) return cudaErrorNotSupported;
     CUtensorMap map;
-    const cuuint64_t gdim[5] = {(cuuint64_t)kC, (cuuint64_t)dm.x, (cuuint64_t)dm.y, (cuuint64_t)dm.z, (cuuint64_t)dm.n};
-    const cuuint64_t gstride[4] = {(cuuint64_t)kC * 2, (cuuint64_t)kC * 2 * dm.x, (cuuint64_t)kC * 2 * dm.x * dm.y,
-                                   (cuuint64_t)kC * 2 * dm.x * dm.y * dm.z};
-    const cuuint32_t box[5] = {(cuuint32_t)kC, (cuuint32_t)g.bx, (cuuint32_t)(g.tall ? g.by + 2 * dil : g.by),
-                               (cuuint32_t)g.bz, 1u};
-    const cuuint32_t estride[5] = {1u, 1u, 1u, 1u, 1u};
-    if (enc(&map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<__nv_bfloat16 *>(x), gdim, gstride, box, estride,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-        return cudaErrorInvalidValue;
+    cudaError_t e = act_map(x, dm, g.bx, g.tall ? g.by + 2 * dil : g.by, g.bz, &map);
+    if (e != cudaSuccess) return e;
 
     int dev = 0, sms = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
     if ((e = cudaFuncSetAttribute(conv_tma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTmSmemMax)) !=
         cudaSuccess)
@@ -953,6 +1173,34 @@ static cudaError_t launch_conv(const __nv_bfloat16 *x, const uint8_t *wimg, cons
     const int nbatch = (g.tiles + kTmTiles - 1) / kTmTiles;
     const int grid = std::max(1, std::min(nbatch, sms));
     conv_tma_kernel<<<grid, kTmThreads, smem, st>>>(map, wimg, bias, mask_act, y, y0, g);
+    return cudaGetLastError();
+}
+
+// Weight gradient on the tensor cores; cudaErrorNotSupported where no tensor
+// copy can address the operands.
+static cudaError_t launch_dw(const __nv_bfloat16 *x, const __nv_bfloat16 *dy, float *dw, Dims dm, int dil, cudaStream_t st) {
+    if ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(dy)) & 15) return cudaErrorNotSupported;
+    DwGeo g;
+    if (!tile_shape(dm, dil, g)) return cudaErrorNotSupported;
+    const int rows = g.by + 2 * dil;
+    g.bstep = g.tall ? dil * g.bx * 128 : 16384;
+    g.xbytes = g.tall ? rows * g.bx * 128 : 3 * 16384;   // whole 1024-byte atoms: bx is a multiple of 8
+    g.stage_bytes = g.xbytes + 16384;
+    g.stages = std::min(kDwMaxStages, (kTmSmemMax - 1024 - (int)sizeof(DwShared)) / g.stage_bytes);
+    if (g.stages < 1) return cudaErrorNotSupported;
+    CUtensorMap mx, md;
+    cudaError_t e = act_map(x, dm, g.bx, g.tall ? rows : g.by, g.bz, &mx);
+    if (e == cudaSuccess) e = act_map(dy, dm, g.bx, g.by, g.bz, &md);
+    if (e != cudaSuccess) return cudaErrorNotSupported;
+    int dev = 0, sms = 0;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(conv_dw_tma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTmSmemMax)) !=
+        cudaSuccess)
+        return e;
+    g.splits = std::max(1, std::min(g.tiles, sms / 9));
+    const size_t smem = 1024 + (size_t)g.stages * g.stage_bytes + sizeof(DwShared);
+    conv_dw_tma_kernel<<<9 * g.splits, kTmThreads, smem, st>>>(mx, md, dw, g);
     return cudaGetLastError();
 }
 
@@ -1073,14 +1321,22 @@ cpmdp_status cpmdp_conv3d_backward_weight(const uint16_t *x, const uint16_t *dy,
     if (s != CPMDP_OK) return s;
     if (!x || !dy || !dw) { set_error("x, dy and dw are required"); return CPMDP_EINVAL; }
     Dims dm{n, z, yy, xx};
-    const int chunk = 512;
-    dim3 grid((dm.nvox() + chunk - 1) / chunk, 27);
-    conv_dw_kernel<<<grid, 256, 0, (cudaStream_t)stream>>>((const __nv_bfloat16 *)x, (const __nv_bfloat16 *)dy, dw, dm,
-                                                          dilation, chunk);
-    CPMDP_CUDA(cudaGetLastError());
+    const __nv_bfloat16 *xb = (const __nv_bfloat16 *)x, *db16 = (const __nv_bfloat16 *)dy;
+    const cudaError_t e = launch_dw(xb, db16, dw, dm, dilation, (cudaStream_t)stream);
+    if (e == cudaErrorNotSupported) {
+        const int chunk = 512;
+        dim3 grid((dm.nvox() + chunk - 1) / chunk, 27);
+        conv_dw_kernel<<<grid, 256, 0, (cudaStream_t)stream>>>(xb, db16, dw, dm, dilation, chunk);
+        CPMDP_CUDA(cudaGetLastError());
+    } else {
+        CPMDP_CUDA(e);
+    }
     if (db) {
-        conv_db_kernel<<<grid_for(dm.nvox(), 64), 256, 0, (cudaStream_t)stream>>>((const __nv_bfloat16 *)dy, db,
-                                                                                    dm.nvox());
+        if (reinterpret_cast<uintptr_t>(dy) & 15)
+            conv_db_kernel<<<grid_for(dm.nvox(), 64), 256, 0, (cudaStream_t)stream>>>(db16, db, dm.nvox());
+        else
+            conv_db_vec_kernel<<<std::min(grid_for(dm.nvox(), 256), 304), 256, 0, (cudaStream_t)stream>>>(
+                reinterpret_cast<const uint4 *>(dy), db, dm.nvox());
         CPMDP_CUDA(cudaGetLastError());
     }
     return CPMDP_OK;
