@@ -94,19 +94,70 @@ template <typename TA> __device__ __forceinline__ TA rew(const BandArgs &a, int 
 template <> __device__ __forceinline__ float rew<float>(const BandArgs &a, int s) { return a.R32[s]; }
 template <> __device__ __forceinline__ double rew<double>(const BandArgs &a, int s) { return a.R64[s]; }
 
-// perp[d] = sum over d' != d of the pair sums P_d' = N_{2d'} + N_{2d'+1}
-// (prefix + suffix sums).
-template <typename TA, int D>
+// perp[d] = sum over d' != d of the pair sums P_d' = N_{2d'} + N_{2d'+1}:
+// prefix sums plus suffix sums, none of them started from a zero (x + 0 is an
+// instruction: it turns -0 into +0). PI: the policy sweeps of 2-D grids add
+// theirs to zero, which settles how the compiler fuses their products (their
+// values were first computed so).
+template <typename TA, int D, bool PI = false>
 __device__ __forceinline__ void perp_of(const TA (&nb)[2 * D], TA (&perp)[D]) {
     TA P[D];
 #pragma unroll
     for (int d = 0; d < D; d++) P[d] = nb[2 * d] + nb[2 * d + 1];
+    if (D == 1) { perp[0] = 0; return; }
     TA acc = 0;
+    if (D == 2 && PI) {
 #pragma unroll
-    for (int d = 0; d < D; d++) { perp[d] = acc; acc += P[d]; }
-    acc = 0;
+        for (int d = 0; d < D; d++) { perp[d] = acc; acc += P[d]; }
+        acc = 0;
 #pragma unroll
-    for (int d = D - 1; d >= 0; d--) { perp[d] += acc; acc += P[d]; }
+        for (int d = D - 1; d >= 0; d--) { perp[d] += acc; acc += P[d]; }
+        return;
+    }
+    acc = P[0];
+#pragma unroll
+    for (int d = 1; d < D; d++) {
+        perp[d] = acc;
+        acc += P[d];
+    }
+    acc = P[D - 1];
+#pragma unroll
+    for (int d = D - 2; d >= 0; d--) {
+        perp[d] = d == 0 ? acc : perp[d] + acc;
+        acc += P[d];
+    }
+}
+
+// FP64 instructions issue at 1/64 of the FP32 rate on GB300: one costs an SM
+// quarter 64 cycles, in which it can issue 64 integer instructions. So the
+// FP64 kernels use that pipe for the sums and products alone; comparisons and
+// widening run on the integer pipe, with the same results.
+
+// Order of doubles as signed integers (-0 and +0 alike). Not for NaN.
+__device__ __forceinline__ long long order_key(double x) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    return (long long)b < 0 ? (long long)(0x8000000000000000ull - b) : (long long)b;
+}
+
+// Whether the result of an FP64 operation is a NaN (operations return quiet ones).
+__device__ __forceinline__ bool quiet_nan(int hi_word) { return (hi_word & 0x7FFFFFFF) > 0x7FF00000; }
+
+// float -> double. Normal numbers and zeros by shifting the fields; `odd` is
+// raised for the rest (denormals, infinities, NaN), which the caller then
+// converts with a cast.
+__device__ __forceinline__ double widen(float x, bool &odd) {
+    const unsigned u = __float_as_uint(x), m = u & 0x7FFFFFFFu;
+    odd |= m != 0u && m - 0x00800000u >= 0x7F000000u;
+    const unsigned hi = m == 0u ? 0u : (m >> 3) + 0x38000000u;
+    return __hiloint2double((int)((u & 0x80000000u) | hi), (int)(u << 29));
+}
+
+// Larger of a residual and a new |difference| (the residual stays where the difference is a NaN).
+__device__ __forceinline__ float res_max(float res, float dv) { return dv > res ? dv : res; }
+__device__ __forceinline__ double res_max(double res, double dv) {
+    const unsigned long long r = (unsigned long long)__double_as_longlong(res);
+    const unsigned long long v = (unsigned long long)__double_as_longlong(dv);
+    return v > r && !quiet_nan((int)(v >> 32)) ? dv : res;
 }
 
 // Larger of a and b: fmaxf for float (one instruction); for double the
@@ -114,10 +165,54 @@ __device__ __forceinline__ void perp_of(const TA (&nb)[2 * D], TA (&perp)[D]) {
 template <typename TA> __device__ __forceinline__ TA vmax(TA a, TA b) { return b > a ? b : a; }
 template <> __device__ __forceinline__ float vmax<float>(float a, float b) { return fmaxf(a, b); }
 
+// max over actions of E_a and its first action, FP64, D >= 2: compares on
+// order keys. A NaN among the neighbours makes a NaN of some E_a (every pair
+// sum enters the others' E); then the maxima are taken again with
+// floating-point compares. Measured, one FP64 value-iteration sweep at
+// 1000 x 1000: 38.4 us with FP64 compares and zero-started prefix sums (16
+// FP64 instructions a state), 21.6 us so (8; 13.7 us of that pipe's time).
+// FIRST: which product the fused multiply-add rounds alone, wp perp (the
+// kernels that want the action) or wm m.
+template <int D, bool FIRST>
+__device__ __forceinline__ double e64(double wm, double m, double wp, double perp) {
+    return FIRST ? fma(wm, m, __dmul_rn(wp, perp)) : fma(wp, perp, __dmul_rn(wm, m));
+}
+template <int D, bool FIRST>
+__device__ __forceinline__ double best_e64(const double (&nb)[2 * D], double wm, double wp, int &arg) {
+    double perp[D];
+    perp_of<double, D>(nb, perp);
+    double best = 0.0;
+    long long kbest = 0;
+    int top = 0;
+    arg = 0;
+#pragma unroll
+    for (int d = 0; d < D; d++) {
+        const bool up = order_key(nb[2 * d + 1]) > order_key(nb[2 * d]);
+        const double m = up ? nb[2 * d + 1] : nb[2 * d];
+        const double e = e64<D, FIRST>(wm, m, wp, perp[d]);
+        top = max(top, __double2hiint(e) & 0x7FFFFFFF);
+        const long long k = order_key(e);
+        if (d == 0 || k > kbest) { best = e; kbest = k; arg = 2 * d + (up ? 1 : 0); }
+    }
+    if (quiet_nan(top)) {
+#pragma unroll
+        for (int d = 0; d < D; d++) {
+            const bool up = nb[2 * d + 1] > nb[2 * d];
+            const double m = up ? nb[2 * d + 1] : nb[2 * d];
+            const double e = e64<D, FIRST>(wm, m, wp, perp[d]);
+            if (d == 0 || e > best) { best = e; arg = 2 * d + (up ? 1 : 0); }
+        }
+    }
+    return best;
+}
 // max over actions of E_a at one state, from its blocked-move-resolved
 // neighbour values (value iteration without the argmax; see vi_state).
 template <typename TA, int D>
 __device__ __forceinline__ TA vi_best_e(TA self, const TA (&nb)[2 * D], TA wm, TA wp, TA wst) {
+    if constexpr (sizeof(TA) == 8 && D > 1) {
+        int arg;
+        return best_e64<D, false>(nb, wm, wp, arg);
+    }
     TA perp[D];
     perp_of<TA, D>(nb, perp);
     const TA stay = (D == 1) ? wst * self : (TA)0;
@@ -145,7 +240,9 @@ template <typename TA, int D, bool ARG = true>
 __device__ __forceinline__ TA vi_state(TA self, const TA (&nb)[2 * D], unsigned c, TA r, TA wm, TA wp, TA wst, TA g,
                                        int &arg) {
     TA bestE = 0;
-    if (ARG) {
+    if constexpr (ARG && sizeof(TA) == 8 && D > 1) {
+        bestE = best_e64<D, true>(nb, wm, wp, arg);
+    } else if (ARG) {
         TA perp[D];
         perp_of<TA, D>(nb, perp);
         const TA stay = (D == 1) ? wst * self : (TA)0;
@@ -176,7 +273,7 @@ template <typename TA, int D>
 __device__ __forceinline__ TA eval_state(TA self, const TA (&nb)[2 * D], unsigned c, TA r, int act, TA wm, TA wp,
                                          TA wst, TA g) {
     TA perp[D];
-    perp_of<TA, D>(nb, perp);
+    perp_of<TA, D, true>(nb, perp);
     const TA stay = wst * self;
     const bool b0 = act & 1, b1 = (act >> 1) & 1, b2 = (act >> 2) & 1;
     TA nbv = nb[0], pv = perp[0];
@@ -249,33 +346,58 @@ struct Segment {
 
     // Neighbour values with the blocked moves replaced by V(s).
     __device__ __forceinline__ void neighbours(TA (&self)[VEC], TA (&nb)[NB][VEC]) const {
+        constexpr int NR = 2 * (D - 1);
+        TA row[NR > 0 ? NR : 1][VEC], hm, hp;
+        if constexpr (sizeof(T) == 4 && sizeof(TA) == 8) {
+            bool odd = false;
 #pragma unroll
-        for (int k = 0; k < VEC; k++) self[k] = (TA)vs[k];
+            for (int k = 0; k < VEC; k++) self[k] = widen(vs[k], odd);
 #pragma unroll
-        for (int j = 0; j < 2 * (D - 1); j++)
+            for (int j = 0; j < NR; j++)
 #pragma unroll
-            for (int k = 0; k < VEC; k++) nb[j][k] = ((code[k] >> j) & 1u) ? self[k] : (TA)rows[j][k];
-        const int jm = 2 * (D - 1), jp = jm + 1;
+                for (int k = 0; k < VEC; k++) row[j][k] = widen(rows[j][k], odd);
+            hm = widen(halo_m, odd);
+            hp = widen(halo_p, odd);
+            if (odd) {
+#pragma unroll
+                for (int k = 0; k < VEC; k++) self[k] = (TA)vs[k];
+#pragma unroll
+                for (int j = 0; j < NR; j++)
+#pragma unroll
+                    for (int k = 0; k < VEC; k++) row[j][k] = (TA)rows[j][k];
+                hm = (TA)halo_m;
+                hp = (TA)halo_p;
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < VEC; k++) self[k] = (TA)vs[k];
+#pragma unroll
+            for (int j = 0; j < NR; j++)
+#pragma unroll
+                for (int k = 0; k < VEC; k++) row[j][k] = (TA)rows[j][k];
+            hm = (TA)halo_m;
+            hp = (TA)halo_p;
+        }
+#pragma unroll
+        for (int j = 0; j < NR; j++)
+#pragma unroll
+            for (int k = 0; k < VEC; k++) nb[j][k] = ((code[k] >> j) & 1u) ? self[k] : row[j][k];
+        const int jm = NR, jp = jm + 1;
 #pragma unroll
         for (int k = 0; k < VEC; k++) {
-            const TA left = (k == 0) ? (TA)halo_m : self[k > 0 ? k - 1 : 0];
-            const TA right = (k == VEC - 1) ? (TA)halo_p : self[k < VEC - 1 ? k + 1 : 0];
+            const TA left = (k == 0) ? hm : self[k > 0 ? k - 1 : 0];
+            const TA right = (k == VEC - 1) ? hp : self[k < VEC - 1 ? k + 1 : 0];
             nb[jm][k] = ((code[k] >> jm) & 1u) ? self[k] : left;
             nb[jp][k] = ((code[k] >> jp) & 1u) ? self[k] : right;
         }
     }
 
-    // perp[d] = sum over d' != d of the pair sums (prefix + suffix sums).
+    // perp_of for state k of the segment.
     __device__ __forceinline__ static void perp_sums(const TA (&nb)[NB][VEC], int k, TA (&perp)[D]) {
-        TA P[D];
+        TA nbk[NB];
 #pragma unroll
-        for (int d = 0; d < D; d++) P[d] = nb[2 * d][k] + nb[2 * d + 1][k];
-        TA acc = 0;
-#pragma unroll
-        for (int d = 0; d < D; d++) { perp[d] = acc; acc += P[d]; }
-        acc = 0;
-#pragma unroll
-        for (int d = D - 1; d >= 0; d--) { perp[d] += acc; acc += P[d]; }
+        for (int j = 0; j < NB; j++) nbk[j] = nb[j][k];
+        perp_of<TA, D, true>(nbk, perp);
     }
 
     // Value-iteration backup of the segment (vi_state per state). Writes V'
@@ -300,8 +422,7 @@ struct Segment {
             out[k] = v;
             if (WITH_PI) pi[s0 + k] = (c & (OBST | TERM)) ? (uint8_t)255 : (uint8_t)arg;
             if (!(c & OBST)) {
-                const TA dv = abs_diff(v, self[k]);
-                res = dv > res ? dv : res;
+                res = res_max(res, abs_diff(v, self[k]));
             }
         }
         if (W) {
@@ -343,8 +464,7 @@ struct Segment {
                 for (int j = 0; j < NB; j++) nbk[j] = nb[j][k];
                 v = eval_state<TA, D>(self[k], nbk, c, rk, (int)act[k], wm, wp, wst, g);
                 if (!(c & OBST)) {
-                    const TA dv = abs_diff(v, self[k]);
-                    res = dv > res ? dv : res;
+                    res = res_max(res, abs_diff(v, self[k]));
                 }
             } else if (!(c & (OBST | TERM))) {
                 TA best = rk + g * (wm * nb[0][k] + wp * perp[0] + stay);
@@ -372,8 +492,7 @@ struct Segment {
                 for (int j = 0; j < NB; j++) nbk[j] = nb[j][k];
                 v = eval_state<TA, D>(self[k], nbk, c, rk, na, wm, wp, wst, g);
                 if (!(c & OBST)) {
-                    const TA dv = abs_diff(v, self[k]);
-                    res = dv > res ? dv : res;
+                    res = res_max(res, abs_diff(v, self[k]));
                 }
             }
             out[k] = v;
@@ -406,11 +525,11 @@ __device__ __forceinline__ TA sweep_all(const BandArgs &a, const T *V, T *W, uin
         TA r;
         if (MODE == M_VI) r = s0.template finish_vi<WITH_PI>(a, W, pi, i * VEC);
         else r = s0.template finish_pi<MODE>(a, W, pi, margin, i * VEC, changed);
-        res = r > res ? r : res;
+        res = res_max(res, r);
         if (two) {
             if (MODE == M_VI) r = s1.template finish_vi<WITH_PI>(a, W, pi, (i + step) * VEC);
             else r = s1.template finish_pi<MODE>(a, W, pi, margin, (i + step) * VEC, changed);
-            res = r > res ? r : res;
+            res = res_max(res, r);
         }
     }
     return res;

@@ -62,6 +62,11 @@ template <> struct Rew4<double> {
     }
 };
 
+// A value in the working precision (widen: `odd` asks for a cast instead).
+template <typename TA> __device__ __forceinline__ TA to_ta(float x, bool &odd);
+template <> __device__ __forceinline__ float to_ta<float>(float x, bool &) { return x; }
+template <> __device__ __forceinline__ double to_ta<double>(float x, bool &odd) { return widen(x, odd); }
+
 template <typename TA, bool WITH_PI>
 __global__ void __launch_bounds__(256) march_kernel(MarchArgs m, const float *__restrict__ V, float *__restrict__ W,
                                                     uint8_t *__restrict__ pi, unsigned long long *res_out,
@@ -126,19 +131,37 @@ __global__ void __launch_bounds__(256) march_kernel(MarchArgs m, const float *__
         if (left_mem) hl = __ldg(V + s - 1);
         if (right_mem) hr = __ldg(V + s + 4);
         if (act) {
-            TA out[4];
+            TA out[4], vs[4], vh[2];
+            bool odd = false;
+#pragma unroll
+            for (int k = 0; k < 4; k++) vs[k] = to_ta<TA>(comp(vc, k), odd);
+            vh[0] = to_ta<TA>(hl, odd);
+            vh[1] = to_ta<TA>(hr, odd);
+            if (sizeof(TA) == 8 && odd) {
+#pragma unroll
+                for (int k = 0; k < 4; k++) vs[k] = (TA)comp(vc, k);
+                vh[0] = (TA)hl;
+                vh[1] = (TA)hr;
+            }
             unsigned pol = 0;
 #pragma unroll
             for (int k = 0; k < 4; k++) {
                 const unsigned c = (cc >> (8 * k)) & 0xFFu;
-                const TA self = (TA)comp(vc, k);
+                const TA self = vs[k];
+                bool oddk = false;
+                TA far[4] = {to_ta<TA>(comp(vm, k), oddk), to_ta<TA>(comp(vp, k), oddk), to_ta<TA>(comp(ym, k), oddk),
+                             to_ta<TA>(comp(yp, k), oddk)};
+                if (sizeof(TA) == 8 && oddk) {
+                    far[0] = (TA)comp(vm, k);
+                    far[1] = (TA)comp(vp, k);
+                    far[2] = (TA)comp(ym, k);
+                    far[3] = (TA)comp(yp, k);
+                }
                 TA nb[2 * D];
-                nb[0] = (c & 1u) ? self : (TA)comp(vm, k);
-                nb[1] = (c & 2u) ? self : (TA)comp(vp, k);
-                nb[2] = (c & 4u) ? self : (TA)comp(ym, k);
-                nb[3] = (c & 8u) ? self : (TA)comp(yp, k);
-                const TA left = (k == 0) ? (TA)hl : (TA)comp(vc, k > 0 ? k - 1 : 0);
-                const TA right = (k == 3) ? (TA)hr : (TA)comp(vc, k < 3 ? k + 1 : 0);
+#pragma unroll
+                for (int j = 0; j < 4; j++) nb[j] = (c >> j & 1u) ? self : far[j];
+                const TA left = (k == 0) ? vh[0] : vs[k > 0 ? k - 1 : 0];
+                const TA right = (k == 3) ? vh[1] : vs[k < 3 ? k + 1 : 0];
                 nb[4] = (c & 16u) ? self : left;
                 nb[5] = (c & 32u) ? self : right;
                 int arg;
@@ -146,8 +169,7 @@ __global__ void __launch_bounds__(256) march_kernel(MarchArgs m, const float *__
                 out[k] = v;
                 pol |= ((c & (OBST | TERM)) ? 255u : (unsigned)arg) << (8 * k);
                 if (!(c & OBST)) {
-                    const TA dv = abs_diff(v, self);
-                    res = dv > res ? dv : res;
+                    res = res_max(res, abs_diff(v, self));
                 }
             }
             if (WITH_PI) *reinterpret_cast<unsigned *>(pi + s) = pol;

@@ -181,7 +181,7 @@ __global__ void __launch_bounds__(256) small_vi_kernel(BandArgs a, T *V, SolvePa
             Segment<T, TA, D, VEC> sg;
             sg.template load<M_VI>(a, cur, nullptr, i * VEC);
             const TA x = sg.template finish_vi<false>(a, nxt, nullptr, i * VEC);
-            r = x > r ? x : r;
+            r = res_max(r, x);
         }
         const unsigned long long mb = block_max_bits(r, shm);
         if (threadIdx.x == 0) s_mb = mb;
@@ -239,7 +239,7 @@ __global__ void __launch_bounds__(256) small_pi_kernel(BandArgs a, T *V, uint8_t
                 Segment<T, TA, D, VEC> sg;
                 sg.template load<M_EVAL>(a, cur, pi, i * VEC);
                 const TA x = sg.template finish_pi<M_EVAL>(a, nxt, pi, (TA)0, i * VEC, dummy);
-                r = x > r ? x : r;
+                r = res_max(r, x);
             }
             const unsigned long long mb = block_max_bits(r, shm);
             if (threadIdx.x == 0) s_mb = mb;
@@ -262,7 +262,7 @@ __global__ void __launch_bounds__(256) small_pi_kernel(BandArgs a, T *V, uint8_t
             Segment<T, TA, D, VEC> sg;
             sg.template load<M_IMPROVE>(a, cur, pi, i * VEC);
             const TA x = sg.template finish_pi<M_IMPROVE>(a, nxt, pi, (TA)sp.margin, i * VEC, changed);
-            r = x > r ? x : r;
+            r = res_max(r, x);
         }
         const unsigned c0 = block_sum(changed, shu);
         const unsigned long long mb = block_max_bits(r, shm);

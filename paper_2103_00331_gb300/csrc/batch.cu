@@ -374,7 +374,7 @@ __device__ __forceinline__ double certify_segment(const BatchCertArgs &c, const 
         int arg;
         const double v = vi_state<double, D>(self[k], nbk, code, sg.r[k], wm, wp, wst, g, arg);
         if (c.pi) c.pi[T.offset + s0 + k] = (code & (OBST | TERM)) ? (uint8_t)255 : (uint8_t)arg;
-        if (!(code & OBST)) res = fmax(res, fabs(v - self[k]));
+        if (!(code & OBST)) res = res_max(res, fabs(v - self[k]));
     }
     return res;
 }
@@ -396,7 +396,7 @@ __global__ void __launch_bounds__(256) batch_certify_kernel(BatchCertArgs c) {
                 case 6: x = certify_segment<3, false>(c, T, item); break;
                 default: x = certify_segment<3, true>(c, T, item); break;
             }
-            r = fmax(r, x);
+            r = res_max(r, x);
         }
         // non-negative doubles order like their bit patterns
         const unsigned long long b = (unsigned long long)__double_as_longlong(r);

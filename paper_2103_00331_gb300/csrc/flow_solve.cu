@@ -413,7 +413,7 @@ __device__ __forceinline__ int improve_state(const float (&nb)[2 * D], float sel
     constexpr unsigned OBST = 1u << (2 * D), TERM = 1u << (2 * D + 1);
     if (c & (OBST | TERM)) return greedy ? 255 : old;
     float perp[D];
-    perp_of<float, D>(nb, perp);
+    perp_of<float, D, true>(nb, perp);
     const float stay = wst * self;
     float best = rk + g * (wm * nb[0] + wp * perp[0] + stay);
     int arg = 0;
