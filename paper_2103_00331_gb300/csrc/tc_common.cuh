@@ -69,6 +69,26 @@ __device__ __forceinline__ void mma(uint32_t d_tmem, uint64_t a, uint64_t b, uin
         "l"(a), "l"(b), "r"(idesc), "r"(accumulate));
 }
 
+// One MMA issued by the thread of the warp whose `lead` is set, in code that
+// the whole warp runs. The instruction takes its operands from uniform
+// registers: where one thread alone runs the loop (inside `if (lane == 0)`),
+// every descriptor is worked out in ordinary registers and moved over, about
+// 125 cycles for an MMA that the tensor cores finish in 50.
+__device__ __forceinline__ void mma_lead(bool lead, uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc,
+                                         uint32_t accumulate) {
+    asm volatile(
+        "{\n.reg .pred p, q;\nsetp.ne.b32 p, %4, 0;\nsetp.ne.b32 q, %5, 0;\n"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
+        "l"(a), "l"(b), "r"(idesc), "r"(accumulate), "r"((uint32_t)lead));
+}
+
+// One thread of the (converged) warp.
+__device__ __forceinline__ bool elect_lead() {
+    uint32_t is;
+    asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xFFFFFFFF;\nselp.u32 %0, 1, 0, p;\n}\n" : "=r"(is));
+    return is != 0;
+}
+
 // D (+)= A * B^T for 128 x 64 (A) and 64 x 64 (B) K-major tiles with K = 64,
 // as BF16x3: A_hi B_hi + A_hi B_lo + A_lo B_hi (4 K-steps of 16 each).
 // Issued by one thread. accumulate = 0 starts D from zero.
@@ -99,6 +119,14 @@ __device__ __forceinline__ void mma_bf16x3_amn(uint32_t d_tmem, uint32_t a_hi, u
 __device__ __forceinline__ void commit(uint64_t *mbar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(mbar))
                  : "memory");
+}
+
+__device__ __forceinline__ void commit_lead(bool lead, uint64_t *mbar) {
+    asm volatile(
+        "{\n.reg .pred q;\nsetp.ne.b32 q, %1, 0;\n"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(smem_u32(mbar)),
+        "r"((uint32_t)lead)
+        : "memory");
 }
 
 __device__ __forceinline__ void mbar_init(uint64_t *mbar, uint32_t count) {
@@ -147,6 +175,31 @@ __device__ __forceinline__ void tma_load_5d(uint32_t dst, const void *tmap, int 
         "%6}], [%7];" ::"r"(dst),
         "l"(tmap), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "r"(smem_u32(mbar))
         : "memory");
+}
+
+// The copies and the expect below, issued by the thread whose `lead` is set in
+// code that the whole warp runs (see mma_lead).
+__device__ __forceinline__ void bulk_g2s_lead(bool lead, uint32_t dst, const void *src, uint32_t bytes, uint64_t *mbar) {
+    asm volatile(
+        "{\n.reg .pred q;\nsetp.ne.b32 q, %4, 0;\n"
+        "@q cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n}\n" ::"r"(dst),
+        "l"(src), "r"(bytes), "r"(smem_u32(mbar)), "r"((uint32_t)lead)
+        : "memory");
+}
+__device__ __forceinline__ void tma_load_5d_lead(bool lead, uint32_t dst, const void *tmap, int c0, int c1, int c2, int c3,
+                                                 int c4, uint64_t *mbar) {
+    asm volatile(
+        "{\n.reg .pred q;\nsetp.ne.b32 q, %8, 0;\n"
+        "@q cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5, "
+        "%6}], [%7];\n}\n" ::"r"(dst),
+        "l"(tmap), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "r"(smem_u32(mbar)), "r"((uint32_t)lead)
+        : "memory");
+}
+__device__ __forceinline__ void mbar_expect_tx_lead(bool lead, uint64_t *mbar, uint32_t bytes) {
+    asm volatile("{\n.reg .pred q;\nsetp.ne.b32 q, %2, 0;\n@q mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n}\n" ::"r"(
+                     smem_u32(mbar)),
+                 "r"(bytes), "r"((uint32_t)lead)
+                 : "memory");
 }
 
 // Arrive on the mbarrier and expect `bytes` of transactions in this phase.

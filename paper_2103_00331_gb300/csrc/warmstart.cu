@@ -119,6 +119,36 @@ __device__ __forceinline__ bool tm_wait(uint64_t *bar, uint32_t phase, volatile 
     return true;
 }
 
+// The same for a whole warp, which then goes on together.
+__device__ __forceinline__ bool tm_wait_warp(uint64_t *bar, uint32_t phase, volatile int *abort) {
+    return __all_sync(0xFFFFFFFFu, tm_wait(bar, phase, abort));
+}
+
+// A tile's place in the grid of tiles, stepped without dividing.
+struct TileAt {
+    int ix, iy, iz, n;
+    template <typename Geo>
+    __device__ __forceinline__ void set(const Geo &g, int tile) {
+        ix = tile % g.tx; tile /= g.tx;
+        iy = tile % g.ty; tile /= g.ty;
+        iz = tile % g.tz;
+        n = tile / g.tz;
+    }
+    template <typename Geo>
+    __device__ __forceinline__ void add(const Geo &g, const TileAt &d) {
+        ix += d.ix;
+        int c = ix >= g.tx;
+        ix -= c ? g.tx : 0;
+        iy += d.iy + c;
+        c = iy >= g.ty;
+        iy -= c ? g.ty : 0;
+        iz += d.iz + c;
+        c = iz >= g.tz;
+        iz -= c ? g.tz : 0;
+        n += d.n + c;
+    }
+};
+
 template <typename Geo>
 __device__ __forceinline__ void tile_origin(const Geo &g, int tile, int &nn, int &x0, int &y0, int &z0) {
     int r = tile;
@@ -142,7 +172,7 @@ __global__ void __launch_bounds__(kTmThreads, 1) conv_tma_kernel(const __grid_co
     uint8_t *sB = sm;
     uint8_t *sA = sm + kTmBStages * kTmBStage;
     TmShared &S = *reinterpret_cast<TmShared *>(sA + (size_t)g.stages * g.stage_bytes);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = tid >> 5;
     if (tid == 0) {
         for (int i = 0; i < g.stages; i++) {
             tc::mbar_init(&S.afull[i], 1);
@@ -170,110 +200,119 @@ __global__ void __launch_bounds__(kTmThreads, 1) conv_tma_kernel(const __grid_co
     const int d = g.dil, sg = g.sign;
 
     if (warp == 4) {
-        if (lane == 0) {
-            // producer: weight tiles per tap group, input boxes per tile and group
-            int alast[kTmMaxStages], blast[kTmBStages];
-            for (int i = 0; i < kTmMaxStages; i++) alast[i] = -1;
-            for (int i = 0; i < kTmBStages; i++) blast[i] = -1;
-            uint32_t acount = 0, gcount = 0;
-            bool ok = true;
-            for (int b = blockIdx.x; ok && b < nbatch; b += gridDim.x) {
-                for (int grp = 0; ok && grp < 9; grp++) {
-                    const int oz = grp / 3 - 1, ox = grp % 3 - 1;
-                    const int bs = (int)(gcount % kTmBStages);
-                    const uint32_t bph = (gcount / kTmBStages) & 1;
-                    if (gcount >= kTmBStages && !tm_wait(&S.bempty[bs], bph ^ 1u, abort)) { ok = false; break; }
-                    tc::mbar_expect_tx(&S.bfull[bs], kTmBStage);
-                    for (int oy = 0; oy < 3; oy++) {
-                        const int t = (oz + 1) * 9 + oy * 3 + (ox + 1);
-                        tc::bulk_g2s(tc::smem_u32(sB + bs * kTmBStage + oy * kCvBTile), wimg + (size_t)t * kCvBTile,
-                                     kCvBTile, &S.bfull[bs]);
+        // producer: weight tiles per tap group, input boxes per tile and group;
+        // the warp runs the loop together, one thread issues
+        const bool lead = tc::elect_lead();
+        uint32_t as = 0, aph = 1, bs = 0, bph = 1;      // phase to wait for: the first round finds free slots
+        uint32_t atotal = 0, btotal = 0;
+        bool ok = true;
+        const uint32_t a0 = tc::smem_u32(sA), b0 = tc::smem_u32(sB);
+        const uint32_t abytes = g.tall ? (uint32_t)((g.by + 2 * d) * g.bx * 128) : 3u * 128u * 128u;
+        TileAt at, one, hop;
+        at.set(g, blockIdx.x * kTmTiles);
+        one.set(g, 1);
+        hop.set(g, gridDim.x * kTmTiles);
+        for (int b = blockIdx.x; ok && b < nbatch; b += gridDim.x) {
+            const int ntile = min(kTmTiles, g.tiles - b * kTmTiles);
+            TileAt t4[kTmTiles];
+            t4[0] = at;
+#pragma unroll
+            for (int j = 1; j < kTmTiles; j++) {
+                t4[j] = t4[j - 1];
+                t4[j].add(g, one);
+            }
+            at.add(g, hop);
+            for (int grp = 0; ok && grp < 9; grp++) {
+                const int oz = grp / 3 - 1, ox = grp % 3 - 1;
+                if (btotal >= kTmBStages && !tm_wait_warp(&S.bempty[bs], bph, abort)) { ok = false; break; }
+                tc::mbar_expect_tx_lead(lead, &S.bfull[bs], kTmBStage);
+#pragma unroll
+                for (int oy = 0; oy < 3; oy++)
+                    tc::bulk_g2s_lead(lead, b0 + bs * kTmBStage + oy * kCvBTile,
+                                      wimg + (size_t)((oz + 1) * 9 + oy * 3 + (ox + 1)) * kCvBTile, kCvBTile, &S.bfull[bs]);
+                btotal++;
+                if (++bs == kTmBStages) { bs = 0; bph ^= 1; }
+#pragma unroll
+                for (int j = 0; j < kTmTiles; j++) {
+                    if (j >= ntile) break;
+                    if (atotal >= (uint32_t)g.stages && !tm_wait_warp(&S.aempty[as], aph, abort)) { ok = false; break; }
+                    const uint32_t dst = a0 + as * (uint32_t)g.stage_bytes;
+                    const int xs = t4[j].ix * g.bx + sg * d * ox, ys = t4[j].iy * g.by, zs = t4[j].iz * g.bz + sg * d * oz;
+                    tc::mbar_expect_tx_lead(lead, &S.afull[as], abytes);
+                    if (g.tall) {
+                        tc::tma_load_5d_lead(lead, dst, &tmx, 0, xs, ys - d, zs, t4[j].n, &S.afull[as]);
+                    } else {
+#pragma unroll
+                        for (int oy = 0; oy < 3; oy++)
+                            tc::tma_load_5d_lead(lead, dst + oy * 16384u, &tmx, 0, xs, ys + sg * d * (oy - 1), zs, t4[j].n,
+                                                 &S.afull[as]);
                     }
-                    blast[bs] = (int)bph;
-                    gcount++;
-                    for (int j = 0; j < kTmTiles; j++) {
-                        const int tile = b * kTmTiles + j;
-                        if (tile >= g.tiles) break;
-                        int nn, x0, y0t, z0;
-                        tile_origin(g, tile, nn, x0, y0t, z0);
-                        const int as = (int)(acount % (uint32_t)g.stages);
-                        const uint32_t ph = (acount / (uint32_t)g.stages) & 1;
-                        if (acount >= (uint32_t)g.stages && !tm_wait(&S.aempty[as], ph ^ 1u, abort)) { ok = false; break; }
-                        const uint32_t dst = tc::smem_u32(sA + (size_t)as * g.stage_bytes);
-                        const int xs = x0 + sg * d * ox, zs = z0 + sg * d * oz;
-                        if (g.tall) {
-                            tc::mbar_expect_tx(&S.afull[as], (uint32_t)((g.by + 2 * d) * g.bx * 128));
-                            tc::tma_load_5d(dst, &tmx, 0, xs, y0t - d, zs, nn, &S.afull[as]);
-                        } else {
-                            tc::mbar_expect_tx(&S.afull[as], 3u * 128u * 128u);
-                            for (int oy = 0; oy < 3; oy++)
-                                tc::tma_load_5d(dst + oy * 16384u, &tmx, 0, xs, y0t + sg * d * (oy - 1), zs, nn,
-                                                &S.afull[as]);
-                        }
-                        alast[as] = (int)ph;
-                        acount++;
-                    }
+                    atotal++;
+                    if (++as == (uint32_t)g.stages) { as = 0; aph ^= 1; }
                 }
             }
-            // every copy this thread issued lands before the CTA's shared memory goes
-            for (int i = 0; i < g.stages; i++)
-                if (alast[i] >= 0) tc::mbar_wait(&S.afull[i], (uint32_t)alast[i], kCvWaitCycles);
-            for (int i = 0; i < kTmBStages; i++)
-                if (blast[i] >= 0) tc::mbar_wait(&S.bfull[i], (uint32_t)blast[i], kCvWaitCycles);
         }
+        // every copy this warp issued lands before the CTA's shared memory
+        // goes: the last of each slot was copy number total - 1 - back
+        for (uint32_t back = 0; back < min(atotal, (uint32_t)g.stages); back++) {
+            const uint32_t k = atotal - 1 - back;
+            tc::mbar_wait(&S.afull[k % (uint32_t)g.stages], (k / (uint32_t)g.stages) & 1, kCvWaitCycles);
+        }
+        for (uint32_t back = 0; back < min(btotal, (uint32_t)kTmBStages); back++) {
+            const uint32_t k = btotal - 1 - back;
+            tc::mbar_wait(&S.bfull[k % kTmBStages], (k / kTmBStages) & 1, kCvWaitCycles);
+        }
+        __syncwarp();
     } else if (warp == 5) {
-        if (lane == 0) {
-            // MMA issuer
-            uint32_t acount = 0, gcount = 0, bcount = 0;
-            uint64_t *lastbar = nullptr;
-            uint32_t lastph = 0;
-            bool ok = true;
-            for (int b = blockIdx.x; ok && b < nbatch; b += gridDim.x, bcount++) {
-                const int buf = bcount & 1;
-                if (bcount >= 2 && !tm_wait(&S.acce[buf], ((bcount >> 1) - 1) & 1, abort)) { ok = false; break; }
-                tc::fence_after();
-                const uint32_t dacc = tmem + (uint32_t)buf * (kTmCols / 2);
-                for (int grp = 0; ok && grp < 9; grp++) {
-                    const int bs = (int)(gcount % kTmBStages);
-                    const uint32_t bph = (gcount / kTmBStages) & 1;
-                    if (!tm_wait(&S.bfull[bs], bph, abort)) { ok = false; break; }
+        // MMA issuer: the warp runs the loop together, one thread issues
+        const bool lead = tc::elect_lead();
+        uint32_t as = 0, aph = 0, bs = 0, bph = 0, bcount = 0;
+        uint64_t *lastbar = nullptr;
+        uint32_t lastph = 0;
+        bool ok = true;
+        const uint32_t a0 = tc::smem_u32(sA), b0 = tc::smem_u32(sB);
+        const uint32_t ostep = g.tall ? (uint32_t)(sg * d * g.bx * 128) : 16384u;   // from one oy to the next
+        const uint32_t ofirst = g.tall ? (uint32_t)((d - sg * d) * g.bx * 128) : 0u;
+        for (int b = blockIdx.x; ok && b < nbatch; b += gridDim.x, bcount++) {
+            const uint32_t buf = bcount & 1;
+            if (bcount >= 2 && !tm_wait_warp(&S.acce[buf], ((bcount >> 1) - 1) & 1, abort)) { ok = false; break; }
+            tc::fence_after();
+            const uint32_t dacc = tmem + buf * (kTmCols / 2);
+            const int ntile = min(kTmTiles, g.tiles - b * kTmTiles);
+            for (int grp = 0; ok && grp < 9; grp++) {
+                if (!tm_wait_warp(&S.bfull[bs], bph, abort)) { ok = false; break; }
+                const uint64_t bd = tc::sdesc(b0 + bs * kTmBStage);
+                for (int j = 0; j < ntile; j++) {
+                    if (!tm_wait_warp(&S.afull[as], aph, abort)) { ok = false; break; }
                     tc::fence_after();
-                    const uint32_t bb = tc::smem_u32(sB + bs * kTmBStage);
-                    for (int j = 0; j < kTmTiles; j++) {
-                        if (b * kTmTiles + j >= g.tiles) break;
-                        const int as = (int)(acount % (uint32_t)g.stages);
-                        const uint32_t ph = (acount / (uint32_t)g.stages) & 1;
-                        if (!tm_wait(&S.afull[as], ph, abort)) { ok = false; break; }
-                        tc::fence_after();
-                        const uint32_t ab = tc::smem_u32(sA + (size_t)as * g.stage_bytes);
-                        for (int oy = 0; oy < 3; oy++) {
-                            const uint32_t aoff = g.tall ? (uint32_t)((sg * d * (oy - 1) + d) * g.bx * 128)
-                                                         : (uint32_t)(oy * 16384);
+                    const uint64_t ad = tc::sdesc(a0 + as * (uint32_t)g.stage_bytes + ofirst);
+                    const uint32_t dj = dacc + (uint32_t)j * 64u, acc0 = grp > 0 ? 1u : 0u;
 #pragma unroll
-                            for (int ks = 0; ks < 4; ks++)
-                                tc::mma(dacc + (uint32_t)j * 64u, tc::sdesc(ab + aoff + ks * 32),
-                                        tc::sdesc(bb + oy * kCvBTile + ks * 32), tc::kIdescM128N64,
-                                        (grp > 0 || oy > 0 || ks > 0) ? 1u : 0u);
-                        }
-                        tc::commit(&S.aempty[as]);
-                        lastbar = &S.aempty[as];
-                        lastph = ph;
-                        acount++;
-                    }
-                    if (!ok) break;
-                    tc::commit(&S.bempty[bs]);
-                    lastbar = &S.bempty[bs];
-                    lastph = bph;
-                    gcount++;
+                    for (int oy = 0; oy < 3; oy++)
+#pragma unroll
+                        for (int ks = 0; ks < 4; ks++)
+                            tc::mma_lead(lead, dj, ad + (uint64_t)(((int)ostep * oy + ks * 32) >> 4),
+                                         bd + (uint64_t)((oy * kCvBTile + ks * 32) >> 4), tc::kIdescM128N64,
+                                         oy > 0 || ks > 0 ? 1u : acc0);
+                    tc::commit_lead(lead, &S.aempty[as]);
+                    lastbar = &S.aempty[as];
+                    lastph = aph;
+                    if (++as == (uint32_t)g.stages) { as = 0; aph ^= 1; }
                 }
                 if (!ok) break;
-                tc::commit(&S.accf[buf]);
-                lastbar = &S.accf[buf];
-                lastph = (bcount >> 1) & 1;
+                tc::commit_lead(lead, &S.bempty[bs]);
+                lastbar = &S.bempty[bs];
+                lastph = bph;
+                if (++bs == kTmBStages) { bs = 0; bph ^= 1; }
             }
-            // the MMAs complete in order: the last commit covers them all
-            if (lastbar) tc::mbar_wait(lastbar, lastph, kCvWaitCycles);
+            if (!ok) break;
+            tc::commit_lead(lead, &S.accf[buf]);
+            lastbar = &S.accf[buf];
+            lastph = (bcount >> 1) & 1;
         }
+        // the MMAs complete in order: the last commit covers them all
+        if (lastbar) tc::mbar_wait(lastbar, lastph, kCvWaitCycles);
+        __syncwarp();
     } else {
         // epilogue: warps 0-3, thread = tile row = TMEM lane
         const int r = tid;
@@ -382,7 +421,7 @@ __global__ void __launch_bounds__(kTmThreads, 1) conv_dw_tma_kernel(const __grid
     extern __shared__ uint8_t smem_raw[];
     uint8_t *sm = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     DwShared &S = *reinterpret_cast<DwShared *>(sm + (size_t)g.stages * g.stage_bytes);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = tid >> 5;
     const int split = blockIdx.x / 9, oz = (int)(blockIdx.x % 9) / 3 - 1, ox = (int)(blockIdx.x % 3) - 1;
     if (tid == 0) {
         for (int i = 0; i < g.stages; i++) {
@@ -406,58 +445,64 @@ __global__ void __launch_bounds__(kTmThreads, 1) conv_dw_tma_kernel(const __grid
     const int d = g.dil;
 
     if (warp == 4) {
-        if (lane == 0) {
-            int last[kDwMaxStages];
-            for (int i = 0; i < kDwMaxStages; i++) last[i] = -1;
-            uint32_t count = 0;
-            for (int tile = split; tile < g.tiles; tile += g.splits, count++) {
-                const int st = (int)(count % (uint32_t)g.stages);
-                const uint32_t ph = (count / (uint32_t)g.stages) & 1;
-                if (count >= (uint32_t)g.stages && !tm_wait(&S.empty[st], ph ^ 1u, abort)) break;
-                int nn, x0, y0, z0;
-                tile_origin(g, tile, nn, x0, y0, z0);
-                const uint32_t dst = tc::smem_u32(sm + (size_t)st * g.stage_bytes);
-                const int xs = x0 + d * ox, zs = z0 + d * oz;
-                tc::mbar_expect_tx(&S.full[st], (uint32_t)g.xbytes + 16384u);
-                if (g.tall) {
-                    tc::tma_load_5d(dst, &tmx, 0, xs, y0 - d, zs, nn, &S.full[st]);
-                } else {
-                    for (int oy = 0; oy < 3; oy++)
-                        tc::tma_load_5d(dst + (uint32_t)(oy * g.bstep), &tmx, 0, xs, y0 + d * (oy - 1), zs, nn,
-                                        &S.full[st]);
-                }
-                tc::tma_load_5d(dst + (uint32_t)g.xbytes, &tmd, 0, x0, y0, z0, nn, &S.full[st]);
-                last[st] = (int)ph;
+        const bool lead = tc::elect_lead();
+        uint32_t st = 0, ph = 1, total = 0;              // the first round finds free slots
+        const uint32_t s0 = tc::smem_u32(sm);
+        TileAt at, hop;
+        at.set(g, split);
+        hop.set(g, g.splits);
+        for (int tile = split; tile < g.tiles; tile += g.splits) {
+            if (total >= (uint32_t)g.stages && !tm_wait_warp(&S.empty[st], ph, abort)) break;
+            const uint32_t dst = s0 + st * (uint32_t)g.stage_bytes;
+            const int x0 = at.ix * g.bx, y0 = at.iy * g.by, z0 = at.iz * g.bz, xs = x0 + d * ox, zs = z0 + d * oz;
+            tc::mbar_expect_tx_lead(lead, &S.full[st], (uint32_t)g.xbytes + 16384u);
+            if (g.tall) {
+                tc::tma_load_5d_lead(lead, dst, &tmx, 0, xs, y0 - d, zs, at.n, &S.full[st]);
+            } else {
+#pragma unroll
+                for (int oy = 0; oy < 3; oy++)
+                    tc::tma_load_5d_lead(lead, dst + (uint32_t)(oy * g.bstep), &tmx, 0, xs, y0 + d * (oy - 1), zs, at.n,
+                                         &S.full[st]);
             }
-            // every copy this thread issued lands before the CTA's shared memory goes
-            for (int i = 0; i < g.stages; i++)
-                if (last[i] >= 0) tc::mbar_wait(&S.full[i], (uint32_t)last[i], kCvWaitCycles);
+            tc::tma_load_5d_lead(lead, dst + (uint32_t)g.xbytes, &tmd, 0, x0, y0, z0, at.n, &S.full[st]);
+            at.add(g, hop);
+            total++;
+            if (++st == (uint32_t)g.stages) { st = 0; ph ^= 1; }
         }
+        // every copy this warp issued lands before the CTA's shared memory goes
+        for (uint32_t back = 0; back < min(total, (uint32_t)g.stages); back++) {
+            const uint32_t k = total - 1 - back;
+            tc::mbar_wait(&S.full[k % (uint32_t)g.stages], (k / (uint32_t)g.stages) & 1, kCvWaitCycles);
+        }
+        __syncwarp();
     } else if (warp == 5) {
-        if (lane == 0) {
-            uint32_t count = 0;
-            uint64_t *lastbar = nullptr;
-            uint32_t lastph = 0;
-            for (int tile = split; tile < g.tiles; tile += g.splits, count++) {
-                const int st = (int)(count % (uint32_t)g.stages), buf = count & 1;
-                if (count >= 2 && !tm_wait(&S.acce[buf], ((count >> 1) - 1) & 1, abort)) break;
-                if (!tm_wait(&S.full[st], (count / (uint32_t)g.stages) & 1, abort)) break;
-                tc::fence_after();
-                const uint32_t a0 = tc::smem_u32(sm + (size_t)st * g.stage_bytes), b0 = a0 + (uint32_t)g.xbytes;
+        const bool lead = tc::elect_lead();
+        uint32_t count = 0, st = 0, sph = 0;
+        uint64_t *lastbar = nullptr;
+        uint32_t lastph = 0;
+        const uint32_t s0 = tc::smem_u32(sm);
+        for (int tile = split; tile < g.tiles; tile += g.splits, count++) {
+            const uint32_t buf = count & 1;
+            if (count >= 2 && !tm_wait_warp(&S.acce[buf], ((count >> 1) - 1) & 1, abort)) break;
+            if (!tm_wait_warp(&S.full[st], sph, abort)) break;
+            tc::fence_after();
+            const uint32_t a0 = s0 + st * (uint32_t)g.stage_bytes;
+            const uint64_t ad = tc::sdesc_mn(a0, (uint32_t)g.bstep), bd = tc::sdesc_mn(a0 + (uint32_t)g.xbytes, 8192u);
 #pragma unroll
-                for (int i = 0; i < 2; i++)
+            for (int i = 0; i < 2; i++)
 #pragma unroll
-                    for (int ks = 0; ks < 8; ks++)
-                        tc::mma(tmem + 128u * buf + 64u * i, tc::sdesc_mn(a0 + (uint32_t)(i * g.bstep) + ks * 2048u, (uint32_t)g.bstep),
-                                tc::sdesc_mn(b0 + ks * 2048u, 8192u), kDwIdesc, ks > 0 ? 1u : 0u);
-                tc::commit(&S.empty[st]);
-                tc::commit(&S.accf[buf]);
-                lastbar = &S.accf[buf];
-                lastph = (count >> 1) & 1;
-            }
-            // the MMAs complete in order: the last commit covers them all
-            if (lastbar) tc::mbar_wait(lastbar, lastph, kCvWaitCycles);
+                for (int ks = 0; ks < 8; ks++)
+                    tc::mma_lead(lead, tmem + 128u * buf + 64u * i, ad + (uint64_t)((i * g.bstep + ks * 2048) >> 4),
+                                 bd + (uint64_t)(ks * 2048 >> 4), kDwIdesc, ks > 0 ? 1u : 0u);
+            tc::commit_lead(lead, &S.empty[st]);
+            tc::commit_lead(lead, &S.accf[buf]);
+            lastbar = &S.accf[buf];
+            lastph = (count >> 1) & 1;
+            if (++st == (uint32_t)g.stages) { st = 0; sph ^= 1; }
         }
+        // the MMAs complete in order: the last commit covers them all
+        if (lastbar) tc::mbar_wait(lastbar, lastph, kCvWaitCycles);
+        __syncwarp();
     } else {
         const int half = tid >> 6, ci = tid & 63;   // rows of A: 64 of oy = -1 (i = 1: 0), 64 of oy = 0 (1)
         const uint32_t t0 = tmem + ((uint32_t)(32 * warp) << 16);
@@ -669,65 +714,77 @@ __device__ __forceinline__ void coarse_of(const BatchInst &I, int cell, int &cz,
     cz = cell / (xc * yc);
 }
 
-// One thread per coarse cell; rows of the cell whose x extent is a full
-// aligned group of 4 (every row of an instance with x side a multiple of
-// 4) are read as one 16-byte reward load and one 4-byte code load, so
-// neighbouring cells' threads read neighbouring bytes.
-__global__ void features_kernel(const BatchInst *__restrict__ inst, const uint8_t *__restrict__ code,
-                                const float *__restrict__ R, int first, int count, int cells,
-                                __nv_bfloat16 *__restrict__ feat) {
-    const long long total = (long long)count * cells;
-    for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; g < total; g += (long long)gridDim.x * blockDim.x) {
-        const int i = (int)(g / cells), cell = (int)(g % cells);
-        const BatchInst I = inst[first + i];
-        int cz, cy, cx, zc, yc, xc;
-        coarse_of(I, cell, cz, cy, cx, zc, yc, xc);
-        const unsigned ob = 1u << (2 * I.ndim), tb = 1u << (2 * I.ndim + 1);
-        float rsum = 0.f, tmax = 0.f;
-        int live = 0, obst = 0, n = 0, any_t = 0;
-        const int x0 = cx * kF, x1 = min(x0 + kF, I.shape[2]);
-        const bool vec = x1 - x0 == kF && I.shape[2] % 4 == 0 && I.offset % 4 == 0;
-        for (int z = cz * kF; z < min((cz + 1) * kF, I.shape[0]); z++)
-            for (int y = cy * kF; y < min((cy + 1) * kF, I.shape[1]); y++) {
-                const long long row = I.offset + (long long)z * I.stride[0] + y * I.stride[1];
-                float r4[kF];
-                unsigned c4[kF];
-                if (vec) {
-                    const float4 rv = *reinterpret_cast<const float4 *>(R + row + x0);
-                    const unsigned cw = *reinterpret_cast<const unsigned *>(code + row + x0);
-                    r4[0] = rv.x; r4[1] = rv.y; r4[2] = rv.z; r4[3] = rv.w;
+// One thread per coarse cell (blockIdx.y: instances); rows of the cell whose x
+// extent is a full aligned group of 4 (every row of an instance with x side a
+// multiple of 4) are read as one 16-byte reward load and one 4-byte code load,
+// so neighbouring cells' threads read neighbouring bytes. A cell's 128 bytes
+// of channels are written by 8 threads, 16 bytes each, from shared memory: a
+// warp stores whole lines (one thread a cell, 78 us for 128 instances of 64^3;
+// so, 42 us: 168 MB read, 67 MB written).
+constexpr int kFeatThreads = 256;
+
+__global__ void __launch_bounds__(kFeatThreads) features_kernel(const BatchInst *__restrict__ inst,
+                                                                const uint8_t *__restrict__ code,
+                                                                const float *__restrict__ R, int first, int count,
+                                                                int cells, __nv_bfloat16 *__restrict__ feat) {
+    __shared__ uint2 sh[kFeatThreads];
+    const int base = blockIdx.x * kFeatThreads, cell = base + threadIdx.x;
+    for (int i = blockIdx.y; i < count; i += gridDim.y) {
+        if (cell < cells) {
+            const BatchInst I = inst[first + i];
+            int cz, cy, cx, zc, yc, xc;
+            coarse_of(I, cell, cz, cy, cx, zc, yc, xc);
+            const unsigned ob = 1u << (2 * I.ndim), tb = 1u << (2 * I.ndim + 1);
+            float rsum = 0.f, tmax = 0.f;
+            int live = 0, obst = 0, n = 0, any_t = 0;
+            const int x0 = cx * kF, x1 = min(x0 + kF, I.shape[2]);
+            const bool vec = x1 - x0 == kF && I.shape[2] % 4 == 0 && I.offset % 4 == 0;
+            for (int z = cz * kF; z < min((cz + 1) * kF, I.shape[0]); z++)
+                for (int y = cy * kF; y < min((cy + 1) * kF, I.shape[1]); y++) {
+                    const long long row = I.offset + (long long)z * I.stride[0] + y * I.stride[1];
+                    float r4[kF];
+                    unsigned c4[kF];
+                    if (vec) {
+                        const float4 rv = *reinterpret_cast<const float4 *>(R + row + x0);
+                        const unsigned cw = *reinterpret_cast<const unsigned *>(code + row + x0);
+                        r4[0] = rv.x; r4[1] = rv.y; r4[2] = rv.z; r4[3] = rv.w;
 #pragma unroll
-                    for (int k = 0; k < kF; k++) c4[k] = (cw >> (8 * k)) & 0xFFu;
-                } else {
+                        for (int k = 0; k < kF; k++) c4[k] = (cw >> (8 * k)) & 0xFFu;
+                    } else {
+#pragma unroll
+                        for (int k = 0; k < kF; k++) {
+                            const bool in = x0 + k < x1;
+                            r4[k] = in ? R[row + x0 + k] : 0.f;
+                            c4[k] = in ? code[row + x0 + k] : 0xFFFFFFFFu;   // marks "outside the grid"
+                        }
+                    }
 #pragma unroll
                     for (int k = 0; k < kF; k++) {
-                        const bool in = x0 + k < x1;
-                        r4[k] = in ? R[row + x0 + k] : 0.f;
-                        c4[k] = in ? code[row + x0 + k] : 0xFFFFFFFFu;   // marks "outside the grid"
+                        const unsigned c = c4[k];
+                        if (c == 0xFFFFFFFFu) continue;
+                        n++;
+                        if (c & ob) { obst++; continue; }
+                        live++;
+                        rsum += r4[k];
+                        if (c & tb) { tmax = any_t ? fmaxf(tmax, r4[k]) : r4[k]; any_t = 1; }
                     }
                 }
-#pragma unroll
-                for (int k = 0; k < kF; k++) {
-                    const unsigned c = c4[k];
-                    if (c == 0xFFFFFFFFu) continue;
-                    n++;
-                    if (c & ob) { obst++; continue; }
-                    live++;
-                    rsum += r4[k];
-                    if (c & tb) { tmax = any_t ? fmaxf(tmax, r4[k]) : r4[k]; any_t = 1; }
-                }
-            }
-        __nv_bfloat16 *f = feat + g * kC;
-        f[0] = __float2bfloat16_rn(live ? rsum / live : 0.f);
-        f[1] = __float2bfloat16_rn((float)obst / (float)n);
-        f[2] = __float2bfloat16_rn(any_t ? tmax : 0.f);
-        f[3] = __float2bfloat16_rn(-logf(1.f - I.gamma) / 5.f);
-        uint4 *f16 = reinterpret_cast<uint4 *>(f);
+            const __nv_bfloat162 lo = __halves2bfloat162(__float2bfloat16_rn(live ? rsum / live : 0.f),
+                                                         __float2bfloat16_rn((float)obst / (float)n));
+            const __nv_bfloat162 hi = __halves2bfloat162(__float2bfloat16_rn(any_t ? tmax : 0.f),
+                                                         __float2bfloat16_rn(-logf(1.f - I.gamma) / 5.f));
+            sh[threadIdx.x] = make_uint2(*reinterpret_cast<const unsigned *>(&lo), *reinterpret_cast<const unsigned *>(&hi));
+        }
+        __syncthreads();
         // channels 4..63: zero (channel 4 is the coarse value, written later)
-        uint2 *f2 = reinterpret_cast<uint2 *>(f);
-        f2[1] = make_uint2(0u, 0u);
-#pragma unroll
-        for (int j = 1; j < 8; j++) f16[j] = make_uint4(0u, 0u, 0u, 0u);
+        uint4 *out = reinterpret_cast<uint4 *>(feat + ((size_t)i * cells + base) * kC);
+        const int part = min(kFeatThreads, cells - base) * 8;
+        for (int e = threadIdx.x; e < part; e += kFeatThreads) {
+            uint4 v = make_uint4(0u, 0u, 0u, 0u);
+            if ((e & 7) == 0) { v.x = sh[e >> 3].x; v.y = sh[e >> 3].y; }
+            out[e] = v;
+        }
+        __syncthreads();
     }
 }
 
@@ -756,58 +813,9 @@ __global__ void targets_kernel(const BatchInst *__restrict__ inst, const uint8_t
     }
 }
 
-// Trilinear interpolation of a coarse array (plus base, if given) at fine
-// state s of instance I: the coarse values sit at the cell centres, a fine
-// coordinate x at (x + 0.5) / 4 - 0.5 in cell units, clamped to the
+// Interpolation in one dimension: the coarse values sit at the cell centres, a
+// fine coordinate p at (p + 0.5) / 4 - 0.5 in cell units, clamped to the
 // outermost centres.
-struct Interp {
-    int lo[3], hi[3];
-    float t[3];
-    int yc, xc;
-    __device__ void at(const BatchInst &I, int s) {
-        const int z = s / I.stride[0], y = (s / I.stride[1]) % I.shape[1], x = s % I.shape[2];
-        const int nc[3] = {(I.shape[0] + kF - 1) / kF, (I.shape[1] + kF - 1) / kF, (I.shape[2] + kF - 1) / kF};
-        const int pos[3] = {z, y, x};
-        yc = nc[1];
-        xc = nc[2];
-#pragma unroll
-        for (int d = 0; d < 3; d++) {
-            float u = ((float)pos[d] + 0.5f) / (float)kF - 0.5f;
-            u = fminf(fmaxf(u, 0.f), (float)(nc[d] - 1));
-            lo[d] = (int)floorf(u);
-            hi[d] = min(lo[d] + 1, nc[d] - 1);
-            t[d] = u - (float)lo[d];
-        }
-    }
-    __device__ float value(const float *cv, const float *bv) const {
-        float v = 0.f;
-#pragma unroll
-        for (int k = 0; k < 8; k++) {
-            const int cz = (k & 4) ? hi[0] : lo[0], cy = (k & 2) ? hi[1] : lo[1], cx = (k & 1) ? hi[2] : lo[2];
-            const float w = ((k & 4) ? t[0] : 1.f - t[0]) * ((k & 2) ? t[1] : 1.f - t[1]) * ((k & 1) ? t[2] : 1.f - t[2]);
-            const int cell = (cz * yc + cy) * xc + cx;
-            v += w * (cv[cell] + (bv ? bv[cell] : 0.f));
-        }
-        return v;
-    }
-};
-
-// Weight of coarse index c in the interpolation at fine coordinate p of a
-// dimension with nc cells (both corners may be c where the clamp folds them).
-__device__ __forceinline__ float interp_weight(int p, int c, int nc) {
-    float u = ((float)p + 0.5f) / (float)kF - 0.5f;
-    u = fminf(fmaxf(u, 0.f), (float)(nc - 1));
-    const int lo = (int)floorf(u), hi = min(lo + 1, nc - 1);
-    const float t = u - (float)lo;
-    return (lo == c ? 1.f - t : 0.f) + (hi == c ? t : 0.f);
-}
-
-// Coarse estimate (plus base) upsampled to every fine state: free states
-// take the interpolation, terminals R(t), obstacles 0. One thread per group
-// of 4 consecutive states of a row: the z and y weights are set once per
-// row, and rows whose length is a multiple of 4 (16-byte aligned, as every
-// instance starts on a multiple of 4 states) are written with one 16-byte
-// store.
 __device__ __forceinline__ void axis_weights(int p, int nc, int &lo, int &hi, float &t) {
     float u = ((float)p + 0.5f) / (float)kF - 0.5f;
     u = fminf(fmaxf(u, 0.f), (float)(nc - 1));
@@ -816,87 +824,163 @@ __device__ __forceinline__ void axis_weights(int p, int nc, int &lo, int &hi, fl
     t = u - (float)lo;
 }
 
-__global__ void upsample_kernel(const BatchInst *__restrict__ inst, const uint8_t *__restrict__ code,
-                                const float *__restrict__ R, int first, int count, int cells,
-                                const float *__restrict__ coarse, const float *__restrict__ base,
-                                float *__restrict__ V) {
-    const BatchInst I0 = inst[first];
-    const int Z = I0.shape[0], Y = I0.shape[1], X = I0.shape[2];
-    const int nq = (X + 3) / 4;
-    const int zc = (Z + kF - 1) / kF, yc = (Y + kF - 1) / kF, xc = (X + kF - 1) / kF;
-    const long long total = (long long)count * Z * Y * nq;
-    for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; g < total; g += (long long)gridDim.x * blockDim.x) {
-        const int q = (int)(g % nq);
-        const long long row = g / nq;
-        const int y = (int)(row % Y);
-        const long long zr = row / Y;
-        const int z = (int)(zr % Z), i = (int)(zr / Z);
-        const BatchInst I = inst[first + i];
-        const unsigned ob = 1u << (2 * I.ndim), tb = 1u << (2 * I.ndim + 1);
-        int zlo, zhi, ylo, yhi;
-        float tz, ty;
-        axis_weights(z, zc, zlo, zhi, tz);
+// Weight of cell c of nc at its fine coordinate 4 c - 2 + o, 0 <= o < 8: the
+// clamp gives an outermost cell all of the coordinates beyond its centre.
+__device__ __forceinline__ float cell_weight(int o, int c, int nc) {
+    const float w = 0.125f + 0.25f * (float)(o < 4 ? o : 7 - o);
+    return (c == 0 && o < 4) || (c == nc - 1 && o >= 4) ? 1.f : w;
+}
+
+__device__ __forceinline__ float lerp(float a, float b, float t) { return (1.f - t) * a + t * b; }
+
+// Trilinear interpolation of coarse + base at the 4 x 4 states z = 4 cz .. + 3,
+// x = 4 q .. + 3 of one y: they lie between the centres cz - 1, cz, cz + 1 and
+// q - 1, q, q + 1, so 18 cell values, reduced over y, then z, then x, serve all
+// 16 states (state by state: 128 loads and products).
+struct Patch {
+    float c[3][3];             // z, x: coarse + base interpolated in y
+    float tz[4], tx[4];        // weights of the upper centre (1: the lower one is the same)
+    __device__ __forceinline__ static void weights(int c, int nc, float (&t)[4]) {
+        t[0] = c > 0 ? 0.625f : 1.f;
+        t[1] = c > 0 ? 0.875f : 1.f;
+        t[2] = c < nc - 1 ? 0.125f : 0.f;
+        t[3] = c < nc - 1 ? 0.375f : 0.f;
+    }
+    __device__ __forceinline__ void load(int cz, int y, int q, int zc, int yc, int xc, const float *cv, const float *bv) {
+        int ylo, yhi;
+        float ty;
         axis_weights(y, yc, ylo, yhi, ty);
-        const float *cv = coarse + (long long)i * cells;
-        const float *bv = base ? base + (long long)i * cells : nullptr;
-        const long long s0 = I.offset + (long long)z * I.stride[0] + (long long)y * I.stride[1];
-        float out[4];
+        weights(cz, zc, tz);
+        weights(q, xc, tx);
+        const int x[3] = {max(q - 1, 0), q, min(q + 1, xc - 1)}, z[3] = {max(cz - 1, 0), cz, min(cz + 1, zc - 1)};
 #pragma unroll
-        for (int k = 0; k < 4; k++) {
-            const int x = 4 * q + k;
-            out[k] = 0.f;
-            if (x >= X) continue;
-            const unsigned c = code[s0 + x];
-            if (c & ob) continue;
-            if (c & tb) { out[k] = R[s0 + x]; continue; }
-            int xlo, xhi;
-            float tx;
-            axis_weights(x, xc, xlo, xhi, tx);
-            float v = 0.f;
+        for (int m = 0; m < 3; m++) {
+            const int r0 = (z[m] * yc + ylo) * xc, r1 = (z[m] * yc + yhi) * xc;
 #pragma unroll
-            for (int m = 0; m < 8; m++) {
-                const int cz = (m & 4) ? zhi : zlo, cy = (m & 2) ? yhi : ylo, cx = (m & 1) ? xhi : xlo;
-                const float w = ((m & 4) ? tz : 1.f - tz) * ((m & 2) ? ty : 1.f - ty) * ((m & 1) ? tx : 1.f - tx);
-                const int cell = (cz * yc + cy) * xc + cx;
-                v += w * (cv[cell] + (bv ? bv[cell] : 0.f));
+            for (int j = 0; j < 3; j++) {
+                float a = cv[r0 + x[j]], b = cv[r1 + x[j]];
+                if (bv) { a += bv[r0 + x[j]]; b += bv[r1 + x[j]]; }
+                c[m][j] = lerp(a, b, ty);
             }
-            out[k] = v;
         }
-        if (X % 4 == 0) {
-            *reinterpret_cast<float4 *>(V + s0 + 4 * q) = make_float4(out[0], out[1], out[2], out[3]);
-        } else {
+    }
+    // the four states of plane z = 4 cz + h (h known at compile time)
+    __device__ __forceinline__ void row(int h, float (&v)[4]) const {
+        float e[3];
 #pragma unroll
-            for (int k = 0; k < 4; k++)
-                if (4 * q + k < X) V[s0 + 4 * q + k] = out[k];
+        for (int j = 0; j < 3; j++) e[j] = lerp(c[h < 2 ? 0 : 1][j], c[h < 2 ? 1 : 2][j], tz[h]);
+#pragma unroll
+        for (int k = 0; k < 4; k++) v[k] = lerp(e[k < 2 ? 0 : 1], e[k < 2 ? 1 : 2], tx[k]);
+    }
+};
+
+// Coarse estimate (plus base) upsampled to every fine state: free states
+// take the interpolation, terminals R(t), obstacles 0. One thread per patch of
+// 4 planes x 4 consecutive states of a row (blockIdx.y: instances); rows whose
+// length is a multiple of 4 (16-byte aligned, as every instance starts on a
+// multiple of 4 states) are written in 16-byte stores. Bound by the stores (V
+// 4 B, code 1 B a state) and the instructions left; 128 instances of 64^3:
+// 208 us state by state.
+__global__ void __launch_bounds__(256) upsample_kernel(const BatchInst *__restrict__ inst, const uint8_t *__restrict__ code,
+                                                       const float *__restrict__ R, int first, int count, int cells,
+                                                       const float *__restrict__ coarse, const float *__restrict__ base,
+                                                       float *__restrict__ V) {
+    const BatchInst &I0 = inst[first];
+    const int Z = I0.shape[0], Y = I0.shape[1], X = I0.shape[2];
+    const int zc = (Z + kF - 1) / kF, yc = (Y + kF - 1) / kF, xc = (X + kF - 1) / kF;
+    const unsigned g = blockIdx.x * blockDim.x + threadIdx.x;
+    if (g >= (unsigned)zc * Y * xc) return;
+    const unsigned row = g / (unsigned)xc, q = g - row * xc, cz = row / (unsigned)Y, y = row - cz * Y;
+    const unsigned ob = 1u << 6, tb = 1u << 7;   // 3-D codes
+    const bool full = X % 4 == 0;
+    const int live = min(4, X - 4 * (int)q);
+    for (int i = blockIdx.y; i < count; i += gridDim.y) {
+        Patch pt;
+        pt.load((int)cz, (int)y, (int)q, zc, yc, xc, coarse + (long long)i * cells, base ? base + (long long)i * cells : nullptr);
+        const long long at = inst[first + i].offset + (long long)(4 * cz * Y + y) * X + 4 * q;
+        const long long plane = (long long)Y * X;
+#pragma unroll
+        for (int h = 0; h < 4; h++) {
+            if (4 * (int)cz + h >= Z) break;
+            const long long s0 = at + h * plane;
+            unsigned cw = 0;
+            if (full) cw = *reinterpret_cast<const unsigned *>(code + s0);
+            else
+                for (int k = 0; k < 4; k++) cw |= (unsigned)(k < live ? code[s0 + k] : ob) << (8 * k);
+            float v[4];
+            pt.row(h, v);
+#pragma unroll
+            for (int k = 0; k < 4; k++) {
+                const unsigned c = cw >> (8 * k);
+                if (c & ob) v[k] = 0.f;
+                else if (c & tb) v[k] = R[s0 + k];
+            }
+            if (full) {
+                *reinterpret_cast<float4 *>(V + s0) = make_float4(v[0], v[1], v[2], v[3]);
+            } else {
+#pragma unroll
+                for (int k = 0; k < 4; k++)
+                    if (k < live) V[s0 + k] = v[k];
+            }
         }
     }
 }
 
 // Fine-level loss of a coarse estimate: with Vh = upsample(base + pred),
 // r(s) = Vh(s) - Vt(s) on the free states (0 on terminals and obstacles,
-// where the upsampling is exact); loss += sum r^2 * inv.
-__global__ void fine_resid_kernel(const BatchInst *__restrict__ inst, const uint8_t *__restrict__ code, int first,
-                                  int count, int cells, const float *__restrict__ pred,
-                                  const float *__restrict__ base, const float *__restrict__ Vt,
-                                  float *__restrict__ r, float inv, float *loss) {
+// where the upsampling is exact); loss += sum r^2 * inv. Threads as in
+// upsample_kernel. 32 instances of 64^3: 123 us with one state a thread, 20 us
+// so (75 MB).
+__global__ void __launch_bounds__(256) fine_resid_kernel(const BatchInst *__restrict__ inst, const uint8_t *__restrict__ code,
+                                                         int first, int count, int cells, const float *__restrict__ pred,
+                                                         const float *__restrict__ base, const float *__restrict__ Vt,
+                                                         float *__restrict__ r, float inv, float *loss) {
     __shared__ float sh[8];
-    const BatchInst I0 = inst[first];
-    const long long per = I0.nstates;
-    const long long total = (long long)count * per;
+    const BatchInst &I0 = inst[first];
+    const int Z = I0.shape[0], Y = I0.shape[1], X = I0.shape[2];
+    const int zc = (Z + kF - 1) / kF, yc = (Y + kF - 1) / kF, xc = (X + kF - 1) / kF;
+    const unsigned g = blockIdx.x * blockDim.x + threadIdx.x;
+    const unsigned row = g / (unsigned)xc, q = g - row * xc, cz = row / (unsigned)Y, y = row - cz * Y;
+    const bool on = g < (unsigned)zc * Y * xc;
+    const bool full = X % 4 == 0, vt16 = full && (reinterpret_cast<uintptr_t>(Vt) & 15) == 0,
+               r16 = full && (reinterpret_cast<uintptr_t>(r) & 15) == 0;   // a multiple of 4 states an instance
+    const int live = min(4, X - 4 * (int)q);
+    const long long plane = (long long)Y * X, at = (long long)(4 * cz * Y + y) * X + 4 * q;
     float l = 0.f;
-    for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; g < total; g += (long long)gridDim.x * blockDim.x) {
-        const int i = (int)(g / per);
-        const int s = (int)(g % per);
-        const BatchInst I = inst[first + i];
-        const unsigned c = code[I.offset + s];
-        float d = 0.f;
-        if (!(c & (3u << (2 * I.ndim)))) {
-            Interp ip;
-            ip.at(I, s);
-            d = ip.value(pred + (long long)i * cells, base ? base + (long long)i * cells : nullptr) - Vt[I.offset + s];
+    for (int i = blockIdx.y; on && i < count; i += gridDim.y) {
+        Patch pt;
+        pt.load((int)cz, (int)y, (int)q, zc, yc, xc, pred + (long long)i * cells, base ? base + (long long)i * cells : nullptr);
+#pragma unroll
+        for (int h = 0; h < 4; h++) {
+            if (4 * (int)cz + h >= Z) break;
+            const long long s0 = inst[first + i].offset + at + h * plane, o = (long long)i * I0.nstates + at + h * plane;
+            unsigned cw = 0;
+            float vt[4] = {0.f, 0.f, 0.f, 0.f}, d[4];
+            if (full) cw = *reinterpret_cast<const unsigned *>(code + s0);
+            else
+                for (int k = 0; k < 4; k++) cw |= (unsigned)(k < live ? code[s0 + k] : 0x40u) << (8 * k);
+            if (vt16) {
+                const float4 v = *reinterpret_cast<const float4 *>(Vt + s0);
+                vt[0] = v.x; vt[1] = v.y; vt[2] = v.z; vt[3] = v.w;
+            } else {
+#pragma unroll
+                for (int k = 0; k < 4; k++)
+                    if (k < live) vt[k] = Vt[s0 + k];
+            }
+            pt.row(h, d);
+#pragma unroll
+            for (int k = 0; k < 4; k++) {
+                d[k] = (cw >> (8 * k) & 0xC0u) ? 0.f : d[k] - vt[k];
+                l += d[k] * d[k] * inv;
+            }
+            if (r16) {
+                *reinterpret_cast<float4 *>(r + o) = make_float4(d[0], d[1], d[2], d[3]);
+            } else {
+#pragma unroll
+                for (int k = 0; k < 4; k++)
+                    if (k < live) r[o + k] = d[k];
+            }
         }
-        r[g] = d;
-        l += d * d * inv;
     }
     for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xFFFFFFFFu, l, o);
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = l;
@@ -912,29 +996,65 @@ __global__ void fine_resid_kernel(const BatchInst *__restrict__ inst, const uint
 // of the interpolation, dL/dpred(c) = 2 inv sum_s w(s, c) r(s) over the fine
 // states whose interpolation reads cell c (coordinates 4c - 2 .. 4c + 5 in
 // each dimension); written into channel 0 of dy, the other channels 0.
-__global__ void fine_grad_kernel(const BatchInst *__restrict__ inst, int first, int count, int cells,
-                                 const float *__restrict__ r, float inv, __nv_bfloat16 *__restrict__ dy) {
-    const long long total = (long long)count * cells;
-    for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; g < total; g += (long long)gridDim.x * blockDim.x) {
-        const int i = (int)(g / cells), cell = (int)(g % cells);
-        const BatchInst I = inst[first + i];
-        int cz, cy, cx, zc, yc, xc;
-        coarse_of(I, cell, cz, cy, cx, zc, yc, xc);
-        const float *ri = r + (long long)i * I.nstates;
-        float acc = 0.f;
-        for (int z = max(0, kF * cz - 2); z <= min(I.shape[0] - 1, kF * cz + 5); z++) {
-            const float wz = interp_weight(z, cz, zc);
-            if (wz == 0.f) continue;
-            for (int y = max(0, kF * cy - 2); y <= min(I.shape[1] - 1, kF * cy + 5); y++) {
-                const float wzy = wz * interp_weight(y, cy, yc);
-                if (wzy == 0.f) continue;
-                for (int x = max(0, kF * cx - 2); x <= min(I.shape[2] - 1, kF * cx + 5); x++)
-                    acc += wzy * interp_weight(x, cx, xc) * ri[z * I.stride[0] + y * I.stride[1] + x];
+// The interpolation is separable: a block takes one (cz, cy) row of cells of an
+// instance, sums its up to 8 x 8 fine rows into one row of weighted sums (each
+// of 4 groups of threads two of the z planes; consecutive threads consecutive
+// states), then takes each cell's up to 8 terms along x from shared memory, and
+// writes the cells' channels in 16-byte pieces. One thread a cell over its 512
+// states took 173 us for 32 instances of 64^3, this 24 us.
+constexpr int kGradX = 64;                           // threads along x per group
+constexpr int kGradCells = 64;                       // cells of the row at a time
+constexpr int kGradStates = kF * kGradCells + 4;     // the states they read
+__global__ void __launch_bounds__(4 * kGradX) fine_grad_kernel(const BatchInst *__restrict__ inst, int first, int count,
+                                                               int zc, int yc, int xc, const float *__restrict__ r, float inv,
+                                                               __nv_bfloat16 *__restrict__ dy) {
+    __shared__ float part[4][kGradStates], out[kGradCells];
+    const BatchInst &I0 = inst[first];
+    const int Z = I0.shape[0], Y = I0.shape[1], X = I0.shape[2];
+    const int cz = blockIdx.x / yc, cy = blockIdx.x - cz * yc;
+    const int grp = threadIdx.x / kGradX, tx = threadIdx.x - grp * kGradX;
+    for (int i = blockIdx.y; i < count; i += gridDim.y) {
+        const float *ri = r + (long long)i * I0.nstates;
+        for (int c0 = 0; c0 < xc; c0 += kGradCells) {
+            const int nc = min(kGradCells, xc - c0), x0 = kF * c0 - 2;   // part[.][e]: state x0 + e
+            for (int e = tx; e < kF * nc + 4; e += kGradX) {
+                const int x = x0 + e;
+                float acc = 0.f;
+#pragma unroll
+                for (int h = 0; h < 2; h++) {
+                    const int z = kF * cz - 2 + 2 * grp + h;
+                    if (z < 0 || z >= Z || x < 0 || x >= X) continue;
+                    const float wz = cell_weight(2 * grp + h, cz, zc);
+                    float v[8];
+#pragma unroll
+                    for (int j = 0; j < 8; j++) {
+                        const int y = kF * cy - 2 + j;
+                        v[j] = y >= 0 && y < Y ? ri[(z * Y + y) * X + x] : 0.f;
+                    }
+#pragma unroll
+                    for (int j = 0; j < 8; j++) acc += wz * cell_weight(j, cy, yc) * v[j];
+                }
+                part[grp][e] = acc;
+            }
+            __syncthreads();
+            for (int c = threadIdx.x; c < nc; c += blockDim.x) {
+                float acc = 0.f;
+#pragma unroll
+                for (int j = 0; j < 8; j++) {
+                    const int e = kF * c + j, x = x0 + e;
+                    if (x < 0 || x >= X) continue;
+                    acc += cell_weight(j, c0 + c, xc) * ((part[0][e] + part[1][e]) + (part[2][e] + part[3][e]));
+                }
+                out[c] = 2.f * inv * acc;
+            }
+            __syncthreads();
+            uint4 *d = reinterpret_cast<uint4 *>(dy + ((((size_t)i * zc + cz) * yc + cy) * xc + c0) * kC);
+            for (int e = threadIdx.x; e < nc * 8; e += blockDim.x) {
+                uint4 v = make_uint4(0u, 0u, 0u, 0u);
+                if ((e & 7) == 0) v.x = (unsigned)__bfloat16_as_ushort(__float2bfloat16_rn(out[e >> 3]));
+                d[e] = v;
             }
         }
-        __nv_bfloat16 *d = dy + g * kC;
-        d[0] = __float2bfloat16_rn(2.f * inv * acc);
-        for (int ch = 1; ch < kC; ch++) d[ch] = __float2bfloat16_rn(0.f);
     }
 }
 
@@ -950,6 +1070,7 @@ __global__ void fine_grad_kernel(const BatchInst *__restrict__ inst, int first, 
 constexpr int kCoarseThreads = 512;
 constexpr int kMaxCoarseCells = 8192;
 
+template <int N>
 __global__ void __launch_bounds__(kCoarseThreads) coarse_vi_kernel(const BatchInst *__restrict__ inst,
                                                                    const uint8_t *__restrict__ code,
                                                                    const float *__restrict__ R, int first, int cells,
@@ -1029,28 +1150,43 @@ __global__ void __launch_bounds__(kCoarseThreads) coarse_vi_kernel(const BatchIn
         vb[c] = v0;
     }
     __syncthreads();
-    const float wm = I.w_move, wp = I.w_perp, wst = I.w_stay;
+    // Each thread keeps the kinds and rewards of its cells in registers (N
+    // cells, kCoarseThreads apart, so a cell's neighbours are at fixed offsets
+    // from the thread's); the larger of a dimension's two neighbours gives the
+    // larger of its two actions' values (weights >= 0, rounding is monotone).
+    // 128 instances of 64^3: 165 us with every cell's kind, reward and
+    // addresses worked out on each sweep.
+    const float wm = I.w_move, wp = I.w_perp;
+    const int s0 = yc * xc, s1 = xc;
+    float rr[N];
+    unsigned kk[(N + 3) / 4];
+#pragma unroll
+    for (int n = 0; n < (N + 3) / 4; n++) kk[n] = 0;
+#pragma unroll
+    for (int n = 0; n < N; n++) {
+        const int c = tid + n * kCoarseThreads;
+        rr[n] = c < cells ? rsum[c] : 0.f;
+        kk[n / 4] |= (c < cells ? (unsigned)kind[c] : 0x40u) << (8 * (n % 4));
+    }
     float *src = va, *dst = vb;
     for (int sweep = 0; sweep < max_sweeps; sweep++) {
         int open = 0;
-        for (int c = tid; c < cells; c += kCoarseThreads) {
-            const uint8_t k = kind[c];
-            if (k & 0xC0) continue;   // obstacles (0) and terminals (their value) never change
-            const float self = src[c];
-            float nb[6];
-            const int step[3] = {yc * xc, xc, 1};
+        const float *p = src + tid, *zm = p - s0, *zp = p + s0, *ym = p - s1, *yp = p + s1;
+        float *out = dst + tid;
 #pragma unroll
-            for (int d = 0; d < 3; d++) {
-                nb[2 * d] = ((k >> (2 * d)) & 1u) ? self : src[c - step[d]];
-                nb[2 * d + 1] = ((k >> (2 * d + 1)) & 1u) ? self : src[c + step[d]];
-            }
-            const float P0 = nb[0] + nb[1], P1 = nb[2] + nb[3], P2 = nb[4] + nb[5];
-            const float perp[3] = {P1 + P2, P0 + P2, P0 + P1};
-            float best = -INFINITY;
-#pragma unroll
-            for (int j = 0; j < 6; j++) best = fmaxf(best, wm * nb[j] + wp * perp[j / 2] + wst * self);
-            const float v = rsum[c] + gc * best;
-            dst[c] = v;
+        for (int n = 0; n < N; n++) {
+            const unsigned k = kk[n / 4] >> (8 * (n % 4));
+            if (k & 0xC0u) continue;   // obstacles (0) and terminals (their value) never change
+            const int o = n * kCoarseThreads;
+            const float self = p[o];
+            const float n0 = (k & 1u) ? self : zm[o], n1 = (k & 2u) ? self : zp[o], n2 = (k & 4u) ? self : ym[o];
+            const float n3 = (k & 8u) ? self : yp[o], n4 = (k & 16u) ? self : p[o - 1], n5 = (k & 32u) ? self : p[o + 1];
+            const float P0 = n0 + n1, P1 = n2 + n3, P2 = n4 + n5;
+            float best = wm * fmaxf(n0, n1) + wp * (P1 + P2);
+            best = fmaxf(best, wm * fmaxf(n2, n3) + wp * (P0 + P2));
+            best = fmaxf(best, wm * fmaxf(n4, n5) + wp * (P0 + P1));
+            const float v = rr[n] + gc * best;
+            out[o] = v;
             open |= fabsf(v - self) >= tol;
         }
         float *t = src; src = dst; dst = t;
@@ -1222,9 +1358,9 @@ cpmdp_status cpmdp_ws_features(const cpmdp_batch *B, int32_t first, int32_t coun
     int cells = 0;
     cpmdp_status s = batch_range(B, first, count, &cells);
     if (s != CPMDP_OK) return s;
-    const long long n = (long long)count * cells;
-    features_kernel<<<grid_for(n, 256), 256, 0, (cudaStream_t)stream>>>(B->d_inst, B->d_code, B->d_R, first, count,
-                                                                        cells, (__nv_bfloat16 *)feat);
+    const dim3 grid((cells + kFeatThreads - 1) / kFeatThreads, std::min(count, 65535));
+    features_kernel<<<grid, kFeatThreads, 0, (cudaStream_t)stream>>>(B->d_inst, B->d_code, B->d_R, first, count, cells,
+                                                                     (__nv_bfloat16 *)feat);
     CPMDP_CUDA(cudaGetLastError());
     return CPMDP_OK;
 }
@@ -1247,9 +1383,10 @@ cpmdp_status cpmdp_ws_upsample(const cpmdp_batch *B, const float *coarse, const 
     cpmdp_status s = batch_range(B, first, count, &cells);
     if (s != CPMDP_OK) return s;
     const BatchInst &I0 = B->inst[(size_t)first];
-    const long long n = (long long)count * I0.shape[0] * I0.shape[1] * ((I0.shape[2] + 3) / 4);
-    upsample_kernel<<<grid_for(n, 256), 256, 0, (cudaStream_t)stream>>>(B->d_inst, B->d_code, B->d_R, first, count,
-                                                                        cells, coarse, base, V);
+    const long long patches = (long long)((I0.shape[0] + kF - 1) / kF) * I0.shape[1] * ((I0.shape[2] + kF - 1) / kF);
+    const dim3 grid((unsigned)((patches + 255) / 256), (unsigned)std::min(count, 65535));
+    upsample_kernel<<<grid, 256, 0, (cudaStream_t)stream>>>(B->d_inst, B->d_code, B->d_R, first, count, cells, coarse,
+                                                            base, V);
     CPMDP_CUDA(cudaGetLastError());
     return CPMDP_OK;
 }
@@ -1263,12 +1400,15 @@ cpmdp_status cpmdp_ws_fine_loss_grad(const cpmdp_batch *B, const float *V_target
     if (!V_target || !pred || !resid || !dy) { set_error("V_target, pred, resid and dy are required"); return CPMDP_EINVAL; }
     const long long n = (long long)count * B->inst[(size_t)first].nstates;
     const float inv = (float)(1.0 / (double)n);
-    fine_resid_kernel<<<grid_for(n, 256), 256, 0, (cudaStream_t)stream>>>(B->d_inst, B->d_code, first, count, cells,
-                                                                          pred, base, V_target, resid, inv, loss);
+    const BatchInst &I0 = B->inst[(size_t)first];
+    const int zc = (I0.shape[0] + kF - 1) / kF, yc = (I0.shape[1] + kF - 1) / kF, xc = (I0.shape[2] + kF - 1) / kF;
+    const unsigned ny = (unsigned)std::min(count, 65535);
+    const dim3 grid((unsigned)(((long long)zc * I0.shape[1] * xc + 255) / 256), ny);
+    fine_resid_kernel<<<grid, 256, 0, (cudaStream_t)stream>>>(B->d_inst, B->d_code, first, count, cells, pred, base,
+                                                              V_target, resid, inv, loss);
     CPMDP_CUDA(cudaGetLastError());
-    const long long nc = (long long)count * cells;
-    fine_grad_kernel<<<grid_for(nc, 256), 256, 0, (cudaStream_t)stream>>>(B->d_inst, first, count, cells, resid, inv,
-                                                                          (__nv_bfloat16 *)dy);
+    fine_grad_kernel<<<dim3((unsigned)(zc * yc), ny), 4 * kGradX, 0, (cudaStream_t)stream>>>(
+        B->d_inst, first, count, zc, yc, xc, resid, inv, (__nv_bfloat16 *)dy);
     CPMDP_CUDA(cudaGetLastError());
     return CPMDP_OK;
 }
@@ -1284,10 +1424,11 @@ cpmdp_status cpmdp_ws_coarse_vi(const cpmdp_batch *B, int32_t first, int32_t cou
     }
     if (!coarse_v || !(tol > 0.f) || max_sweeps < 1) { set_error("coarse_v, tol > 0 and max_sweeps >= 1 required"); return CPMDP_EINVAL; }
     const size_t smem = (size_t)cells * 13;
-    CPMDP_CUDA(cudaFuncSetAttribute(coarse_vi_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    coarse_vi_kernel<<<count, kCoarseThreads, smem, (cudaStream_t)stream>>>(B->d_inst, B->d_code, B->d_R, first, cells,
-                                                                          tol, max_sweeps, coarse_v,
-                                                                          (__nv_bfloat16 *)feat);
+    const auto kern = cells <= 2 * kCoarseThreads ? coarse_vi_kernel<2> : cells <= 8 * kCoarseThreads
+                                                                            ? coarse_vi_kernel<8> : coarse_vi_kernel<16>;
+    CPMDP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    kern<<<count, kCoarseThreads, smem, (cudaStream_t)stream>>>(B->d_inst, B->d_code, B->d_R, first, cells, tol, max_sweeps,
+                                                                coarse_v, (__nv_bfloat16 *)feat);
     CPMDP_CUDA(cudaGetLastError());
     return CPMDP_OK;
 }
