@@ -429,7 +429,7 @@ __global__ void __launch_bounds__(kBThreads, 2) dense_pass_b(const uint8_t *__re
     uint64_t *full_u = reinterpret_cast<uint64_t *>(sm + kBOffBar + 8);
     uint64_t *mbar = reinterpret_cast<uint64_t *>(sm + kBOffBar + 16);
     uint32_t *tslot = reinterpret_cast<uint32_t *>(sm + kBOffBar + 24);
-    const int tid = threadIdx.x, warp = tid >> 5;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);   // (uniform in the warp)
     if (tid == 0) {
         tc::mbar_init(full_raw, 1);
         tc::mbar_init(full_u, 1);
@@ -507,9 +507,10 @@ __global__ void __launch_bounds__(kBThreads, 2) dense_pass_b(const uint8_t *__re
                 if (!wait_all(full_u, uph, err)) { u_failed = true; alive = false; break; }
                 u_pending = false;
                 const uint32_t u1 = aU, u2 = aU + 2 * kTileBytes;
-                if (tid == 0) {
-                    tc::mma_bf16x3(tmem, aZ, aZ + kPairBytes, u2, u2 + kTileBytes, 0);
-                    tc::commit(mbar);
+                if (warp == 0) {
+                    const bool lead = tc::elect_lead();
+                    tc::mma_bf16x3_lead(lead, tmem, aZ, aZ + kPairBytes, u2, u2 + kTileBytes, 0);
+                    tc::commit_lead(lead, mbar);
                 }
                 if (!wait_all(mbar, mph, err)) { alive = false; break; }
                 tc::fence_after();
@@ -531,9 +532,10 @@ __global__ void __launch_bounds__(kBThreads, 2) dense_pass_b(const uint8_t *__re
                     }
                 }
                 sync_for_async();
-                if (tid == 0) {
-                    tc::mma_bf16x3_amn(tmem + 64, aZ, aZ + kPairBytes, u1, u1 + kTileBytes, r > 0 ? 1u : 0u);
-                    tc::commit(mbar);
+                if (warp == 0) {
+                    const bool lead = tc::elect_lead();
+                    tc::mma_bf16x3_amn_lead(lead, tmem + 64, aZ, aZ + kPairBytes, u1, u1 + kTileBytes, r > 0 ? 1u : 0u);
+                    tc::commit_lead(lead, mbar);
                 }
                 if (!wait_all(mbar, mph, err)) { alive = false; break; }
                 // the factor buffer is free: fetch the next item's factors

@@ -116,6 +116,30 @@ __device__ __forceinline__ void mma_bf16x3_amn(uint32_t d_tmem, uint32_t a_hi, u
     }
 }
 
+// Both run by a whole warp and issued by its lead (see mma_lead).
+__device__ __forceinline__ void mma_bf16x3_lead(bool lead, uint32_t d_tmem, uint32_t a_hi, uint32_t a_lo, uint32_t b_hi,
+                                                uint32_t b_lo, uint32_t accumulate) {
+    const uint64_t ah = sdesc(a_hi), al = sdesc(a_lo), bh = sdesc(b_hi), bl = sdesc(b_lo);
+#pragma unroll
+    for (int ks = 0; ks < 4; ks++) {
+        const uint64_t o = (uint64_t)(ks * 32 >> 4);
+        mma_lead(lead, d_tmem, ah + o, bh + o, kIdescM128N64, ks > 0 ? 1u : accumulate);
+        mma_lead(lead, d_tmem, ah + o, bl + o, kIdescM128N64, 1u);
+        mma_lead(lead, d_tmem, al + o, bh + o, kIdescM128N64, 1u);
+    }
+}
+__device__ __forceinline__ void mma_bf16x3_amn_lead(bool lead, uint32_t d_tmem, uint32_t a_hi, uint32_t a_lo, uint32_t b_hi,
+                                                    uint32_t b_lo, uint32_t accumulate) {
+    const uint64_t ah = sdesc_mn(a_hi, 8192), al = sdesc_mn(a_lo, 8192), bh = sdesc(b_hi), bl = sdesc(b_lo);
+#pragma unroll
+    for (int ks = 0; ks < 4; ks++) {
+        const uint64_t oa = (uint64_t)(ks * 2048 >> 4), ob = (uint64_t)(ks * 32 >> 4);
+        mma_lead(lead, d_tmem, ah + oa, bh + ob, kIdescM128N64AMN, ks > 0 ? 1u : accumulate);
+        mma_lead(lead, d_tmem, ah + oa, bl + ob, kIdescM128N64AMN, 1u);
+        mma_lead(lead, d_tmem, al + oa, bh + ob, kIdescM128N64AMN, 1u);
+    }
+}
+
 __device__ __forceinline__ void commit(uint64_t *mbar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(mbar))
                  : "memory");
