@@ -102,6 +102,7 @@ static void free_device(Factors &F) {
     for (void *p : ptrs)
         if (p && p != F.d_arena) cudaFree(p);
     slab_free(F);
+    pad_free(F);
     // the arena came from the pool: returned in stream order (every call on
     // this object has synchronised with its stream before returning)
     if (F.d_arena) cudaFreeAsync(F.d_arena, 0);
@@ -605,8 +606,23 @@ static cpmdp_status run_solver(const cpmdp_factors *h, cpmdp_precision prec, boo
     Ctrl hc;
     memset(&hc, 0, sizeof(hc));
     bool have_ctrl = false;
+    // FP32 solves of rows that are no multiple of 4 states run on a padded
+    // copy of the grid (where there is memory for one)
+    bool padded = pad_wanted(F, prec, o);
+    if (padded) {
+        cudaMemPool_t pool;
+        CPMDP_CUDA(arena_pool(F.device, &pool));
+        st = pad_prepare(const_cast<Factors &>(F), pool, s);
+        if (st == CPMDP_ENOMEM) padded = false;
+        else if (st != CPMDP_OK) { cudaEventDestroy(e0); cudaEventDestroy(e1); return st; }
+    }
+    const Factors &A = padded ? *F.pad : F;   // what is solved
     if (F.kind == CPMDP_GRIDWORLD) {
-        if (!plain) {
+        if (padded) {
+            CPMDP_CUDA(pad_in(F, (const float *)V, s));
+            st = banded_solve(A, prec, pi_mode, A.pad_V, A.pad_pi, o, s);
+            if (st == CPMDP_OK) CPMDP_CUDA(pad_out(F, (float *)V, pi_mode ? pi : nullptr, s));
+        } else if (!plain) {
             st = banded_solve(F, prec, pi_mode, V, pi, o, s);
         } else {
             if (!F.d_q) {
@@ -632,6 +648,10 @@ static cpmdp_status run_solver(const cpmdp_factors *h, cpmdp_precision prec, boo
             // one FP64 backup into scratch: residual + policy of the returned V
             uint8_t *pout = pi_mode ? nullptr : pi;
             st = banded_backup(F, CPMDP_F64, V, F.d_scratch, pout, cert, s);
+        } else if (padded) {
+            const bool want = !pi_mode && pi;
+            st = banded_certify(A, A.pad_V, want ? A.pad_pi : nullptr, cert, s);
+            if (st == CPMDP_OK && want) CPMDP_CUDA(pad_out(F, nullptr, pi, s));
         } else {
             st = banded_certify(F, (const float *)V, pi_mode ? nullptr : pi, cert, s);
         }
@@ -650,10 +670,10 @@ static cpmdp_status run_solver(const cpmdp_factors *h, cpmdp_precision prec, boo
     cudaEventDestroy(e1);
     const int solver = F.kind != CPMDP_GRIDWORLD ? CPMDP_SOLVER_DENSE
                        : plain ? CPMDP_SOLVER_PLAIN
-                       : F.flow_pending ? CPMDP_SOLVER_BARRIER_FREE
-                       : F.march_pending ? CPMDP_SOLVER_MARCH_GRAPH : CPMDP_SOLVER_GRID_BARRIER;
+                       : A.flow_pending ? CPMDP_SOLVER_BARRIER_FREE
+                       : A.march_pending ? CPMDP_SOLVER_MARCH_GRAPH : CPMDP_SOLVER_GRID_BARRIER;
     if (F.kind == CPMDP_GRIDWORLD && !plain) {
-        st = banded_solve_finished(F, dc, s);
+        st = banded_solve_finished(A, dc, s);
         if (st != CPMDP_OK) return st;
     }
     if (!have_ctrl) {
@@ -661,6 +681,7 @@ static cpmdp_status run_solver(const cpmdp_factors *h, cpmdp_precision prec, boo
     } else {
         hc.certify_residual = dc.certify_residual;
     }
+    if (padded) hc.backups = hc.backups / A.nstates * F.nstates;   // of the real states
     if (dense_cert) hc.certify_residual = dc.certify_residual;
     if (dc.status != 0 && !have_ctrl) {
         set_error("a device-side wait exceeded %.3g s; results are undefined", o.timeout_s);

@@ -145,6 +145,11 @@ struct Factors {
     bool flow_in_arena = false;        // d_flow is part of d_arena (set up by the build)
     unsigned flow_base = 0;            // first tag not written to the rings yet
     bool flow_pending = false;         // a launch whose tags are not accounted for yet
+    // the same grid with its rows padded to whole segments of 4 states, for
+    // FP32 solves of rows that are not (padded.cu); made on the first one
+    Factors *pad = nullptr;
+    float *pad_V = nullptr;            // (of the padded object) values and policy of a solve
+    uint8_t *pad_pi = nullptr;
 };
 
 // Thread-local error message.
@@ -184,6 +189,16 @@ cpmdp_status banded_solve(const Factors &F, cpmdp_precision prec, bool policy_it
 cpmdp_status banded_solve_finished(const Factors &F, const Ctrl &dc, cudaStream_t st);
 cpmdp_status banded_plain_vi(const Factors &F, cpmdp_precision prec, void *V, uint8_t *pi,
                              const SolveOpts &o, Ctrl *host_ctrl, cudaStream_t st);
+
+// padded.cu
+// Whether an FP32 GridWorld solve runs on padded rows, and the padded copy
+// (device buffers from `pool`).
+bool pad_wanted(const Factors &F, cpmdp_precision prec, const SolveOpts &o);
+cpmdp_status pad_prepare(Factors &F, cudaMemPool_t pool, cudaStream_t st);
+void pad_free(Factors &F);
+// Values into the padded copy; values and / or policy (nullable) out of it.
+cudaError_t pad_in(const Factors &F, const float *V, cudaStream_t st);
+cudaError_t pad_out(const Factors &F, float *V, uint8_t *pi, cudaStream_t st);
 
 // dense.cu
 cpmdp_status dense_backup(const Factors &F, cpmdp_precision prec, const void *Vin, void *Vout,
