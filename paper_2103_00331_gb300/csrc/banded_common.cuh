@@ -507,6 +507,10 @@ struct Segment {
     }
 };
 
+// Whether the policy sweeps keep one segment in flight per thread (solve_pi_kernel).
+template <typename T, int D>
+constexpr bool pi_one_segment() { return sizeof(T) == 4 && D == 3; }
+
 // All segments of one sweep, grid-stride, two segments in flight per thread.
 // With a grid of co-resident blocks, the states being worked on at any time
 // form one compact window, so the row neighbours one plane away are still in
@@ -517,9 +521,10 @@ __device__ __forceinline__ TA sweep_all(const BandArgs &a, const T *V, T *W, uin
     const int nitems = a.nstates / VEC;
     const int step = gridDim.x * blockDim.x;
     TA res = 0;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nitems; i += 2 * step) {
+    constexpr bool kOne = MODE != M_VI && pi_one_segment<T, D>();
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nitems; i += kOne ? step : 2 * step) {
         Segment<T, TA, D, VEC> s0, s1;
-        const bool two = i + step < nitems;
+        const bool two = !kOne && i + step < nitems;
         s0.template load<MODE>(a, V, pi, i * VEC);
         if (two) s1.template load<MODE>(a, V, pi, (i + step) * VEC);
         TA r;

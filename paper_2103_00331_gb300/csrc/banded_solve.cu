@@ -64,8 +64,14 @@ __global__ void __launch_bounds__(256) solve_vi_kernel(BandArgs a, T *V, T *Wbuf
     }
 }
 
+// FP32, three dimensions: one segment in flight a thread and three blocks an
+// SM (sweep_all); 145 registers for two segments left one block an SM, 8
+// warps: 60.1 us a sweep at 200 x 208 x 212, 34.7 us so (7.1 and 6.3 us at
+// 101 x 97 x 103). Two segments stay where they are as fast or faster (two
+// dimensions; FP64, whose own pipe is the bound: 25.5 us at 1000 x 1000, 28.1
+// with three blocks).
 template <typename T, int D, int VEC>
-__global__ void __launch_bounds__(256) solve_pi_kernel(BandArgs a, T *V, T *Wbuf, uint8_t *pi, SolveParams sp,
+__global__ void __launch_bounds__(256, pi_one_segment<T, D>() ? 3 : 1) solve_pi_kernel(BandArgs a, T *V, T *Wbuf, uint8_t *pi, SolveParams sp,
                                                        Ctrl *ctrl) {
     typedef T TA;
     __shared__ unsigned shm[64];
