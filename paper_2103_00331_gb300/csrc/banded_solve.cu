@@ -166,7 +166,18 @@ __global__ void __launch_bounds__(256, pi_one_segment<T, D>() ? 3 : 1) solve_pi_
 // taken in shared memory (one block barrier per sweep, no global atomics or
 // control-block round trips). Same per-state arithmetic and stopping rules,
 // so the same values, sweep counts and residuals as the kernels above.
+// A sweep's stop decision is one barrier that ORs the threads' own tests; the
+// largest residual itself is only reduced for the trace and at the end (with a
+// reduction of it per sweep, two barriers more, 10 x 10 took 1.10 us a sweep in
+// FP64 and 0.42 in FP32).
 constexpr int kSmallMaxItems = 256;
+
+// A thread's residual not below tol > 0. For floats: tol rounded up to a float
+// separates the same floats (no conversion on the FP64 pipe).
+__device__ __forceinline__ bool res_open(float r, double tol) { return !(r < __double2float_ru(tol)); }
+__device__ __forceinline__ bool res_open(double r, double tol) {
+    return !below_tol((unsigned long long)__double_as_longlong(r), tol);
+}
 
 template <typename T, int D, int VEC>
 __global__ void __launch_bounds__(256) small_vi_kernel(BandArgs a, T *V, SolveParams sp, Ctrl *ctrl,
@@ -174,31 +185,30 @@ __global__ void __launch_bounds__(256) small_vi_kernel(BandArgs a, T *V, SolvePa
     typedef T TA;
     extern __shared__ __align__(16) unsigned char small_raw[];
     __shared__ unsigned shm[64];
-    __shared__ unsigned long long s_mb;
     T *cur = reinterpret_cast<T *>(small_raw), *nxt = cur + a.nstates;
     const int nitems = a.nstates / VEC;
     for (int i = threadIdx.x; i < a.nstates; i += blockDim.x) cur[i] = V[i];
     __syncthreads();
     int k = 0, converged = 0;
-    unsigned long long last = 0ull;
+    TA r = 0;
     while (k < sp.max_iter) {
-        TA r = 0;
+        r = 0;
         for (int i = threadIdx.x; i < nitems; i += blockDim.x) {
             Segment<T, TA, D, VEC> sg;
             sg.template load<M_VI>(a, cur, nullptr, i * VEC);
             const TA x = sg.template finish_vi<false>(a, nxt, nullptr, i * VEC);
             r = res_max(r, x);
         }
-        const unsigned long long mb = block_max_bits(r, shm);
-        if (threadIdx.x == 0) s_mb = mb;
-        __syncthreads();   // the sweep's writes and its residual, for every thread
-        const unsigned long long m = s_mb;
-        if (trace && threadIdx.x == 0) trace[k] = __longlong_as_double((long long)m);
-        last = m;
+        if (trace) {
+            const unsigned long long mb = block_max_bits(r, shm);
+            if (threadIdx.x == 0) trace[k] = __longlong_as_double((long long)mb);
+        }
         k++;
         T *t = cur; cur = nxt; nxt = t;
-        if (below_tol(m, sp.tol)) { converged = 1; break; }
+        // the sweep's writes and its stop decision, for every thread
+        if (!__syncthreads_or(res_open(r, sp.tol))) { converged = 1; break; }
     }
+    const unsigned long long last = block_max_bits(r, shm);
     for (int i = threadIdx.x; i < a.nstates; i += blockDim.x) V[i] = cur[i];
     if (threadIdx.x == 0) {
         ctrl->iterations = k;
@@ -214,16 +224,14 @@ __global__ void __launch_bounds__(256) small_pi_kernel(BandArgs a, T *V, uint8_t
     extern __shared__ __align__(16) unsigned char small_raw[];
     __shared__ unsigned shm[64];
     __shared__ unsigned shu[32];
-    __shared__ unsigned long long s_mb;
-    __shared__ unsigned s_c;
     T *cur = reinterpret_cast<T *>(small_raw), *nxt = cur + a.nstates;
     const int nitems = a.nstates / VEC;
     for (int i = threadIdx.x; i < a.nstates; i += blockDim.x) cur[i] = V[i];
     __syncthreads();
     int total = 0, round = 0, evals = 0, converged = 0;
     long long backups = 0;
-    unsigned long long last = 0ull;
-    unsigned changed_total = 0, dummy = 0;
+    TA r = 0;
+    unsigned changed_total = 0, dummy = 0;   // (this thread's)
     // initial policy: greedy with respect to the input V
     for (int i = threadIdx.x; i < nitems; i += blockDim.x) {
         Segment<T, TA, D, VEC> sg;
@@ -240,53 +248,41 @@ __global__ void __launch_bounds__(256) small_pi_kernel(BandArgs a, T *V, uint8_t
         const int cap = full ? sp.max_eval_iter : min(sp.partial_eval, sp.max_eval_iter);
         int e = 0, eval_ok = 0;
         while (e < cap) {
-            TA r = 0;
+            r = 0;
             for (int i = threadIdx.x; i < nitems; i += blockDim.x) {
                 Segment<T, TA, D, VEC> sg;
                 sg.template load<M_EVAL>(a, cur, pi, i * VEC);
                 const TA x = sg.template finish_pi<M_EVAL>(a, nxt, pi, (TA)0, i * VEC, dummy);
                 r = res_max(r, x);
             }
-            const unsigned long long mb = block_max_bits(r, shm);
-            if (threadIdx.x == 0) s_mb = mb;
-            __syncthreads();
-            const unsigned long long m = s_mb;
-            last = m;
+            const int open = __syncthreads_or(full && res_open(r, sp.eval_tol));
             e++;
             total++;
             backups += a.nstates;
             T *t = cur; cur = nxt; nxt = t;
             // a capped evaluation runs all its sweeps; one to eval_tol stops there
-            if (full && below_tol(m, sp.eval_tol)) { eval_ok = 1; break; }
+            if (full && !open) { eval_ok = 1; break; }
         }
         evals += e;
         // improvement, and the new policy's first evaluation step V' = Q of
         // the action kept or taken (modified policy iteration)
         unsigned changed = 0;
-        TA r = 0;
+        r = 0;
         for (int i = threadIdx.x; i < nitems; i += blockDim.x) {
             Segment<T, TA, D, VEC> sg;
             sg.template load<M_IMPROVE>(a, cur, pi, i * VEC);
             const TA x = sg.template finish_pi<M_IMPROVE>(a, nxt, pi, (TA)sp.margin, i * VEC, changed);
             r = res_max(r, x);
         }
-        const unsigned c0 = block_sum(changed, shu);
-        const unsigned long long mb = block_max_bits(r, shm);
-        if (threadIdx.x == 0) {
-            s_c = c0;
-            s_mb = mb;
-        }
-        __syncthreads();   // the policy changes, their count and V', for every thread
-        const unsigned c = s_c;
-        const unsigned long long m = s_mb;
-        last = m;
-        changed_total += c;
+        const int open = __syncthreads_or(res_open(r, sp.eval_tol));
+        const int moved = __syncthreads_or(changed > 0);   // the policy changes and V', for every thread
+        changed_total += changed;
         total++;
         round++;
         backups += (long long)a.nstates * sp.nactions;
         T *t = cur; cur = nxt; nxt = t;
-        if (c == 0) {
-            if (below_tol(m, sp.eval_tol)) { converged = 1; break; }   // stable policy, V' within eval_tol
+        if (!moved) {
+            if (!open) { converged = 1; break; }   // stable policy, V' within eval_tol
             if (!eval_ok) {
                 if (full) break;   // the evaluation limit ran out
                 full = true;       // evaluate this policy to eval_tol before deciding
@@ -295,6 +291,8 @@ __global__ void __launch_bounds__(256) small_pi_kernel(BandArgs a, T *V, uint8_t
         }
         if (!eval_ok && full) break;
     }
+    const unsigned long long last = block_max_bits(r, shm);
+    const unsigned changes = block_sum(changed_total, shu);
     for (int i = threadIdx.x; i < a.nstates; i += blockDim.x) V[i] = cur[i];
     if (threadIdx.x == 0) {
         ctrl->rounds = round;
@@ -303,7 +301,7 @@ __global__ void __launch_bounds__(256) small_pi_kernel(BandArgs a, T *V, uint8_t
         ctrl->converged = converged;
         ctrl->last_residual = __longlong_as_double((long long)last);
         ctrl->backups = backups;
-        ctrl->changed_total = changed_total;
+        ctrl->changed_total = changes;
     }
 }
 
@@ -374,9 +372,12 @@ static cudaError_t solve_t(const Factors &F, bool pim, T *V, uint8_t *pi, const 
     const int vec = band_pick_vec(F, sizeof(T), V, W);
     constexpr int V2 = (int)(16 / sizeof(T));
     cudaError_t e = cudaErrorInvalidValue;
-    // one block's worth of segments, values within the default 48 KB of shared memory
+    // one block's worth of segments, values within the default 48 KB of shared
+    // memory. FP64 grids of up to 256 states take one state a thread: a warp
+    // gets a quarter of the SM's FP64 rate, so more warps of fewer states are
+    // faster (10 x 10: 1.13 us a sweep with two states a thread).
     if (small_ok && F.nstates / vec <= kSmallMaxItems && 2 * (size_t)F.nstates * sizeof(T) <= 48 * 1024) {
-        if (vec == 1) { CPMDP_DISPATCH_D(F.ndim, e = (launch_small<T, DD, 1>(F, pim, V, pi, sp, trace, st))); }
+        if (vec == 1 || (sizeof(T) == 8 && F.nstates <= kSmallMaxItems)) { CPMDP_DISPATCH_D(F.ndim, e = (launch_small<T, DD, 1>(F, pim, V, pi, sp, trace, st))); }
         else { CPMDP_DISPATCH_D(F.ndim, e = (launch_small<T, DD, V2>(F, pim, V, pi, sp, trace, st))); }
         return e;
     }
