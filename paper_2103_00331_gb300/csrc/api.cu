@@ -93,6 +93,34 @@ static cudaError_t arena_pool(int device, cudaMemPool_t *out) {
     return cudaSuccess;
 }
 
+// What a solve call needs on the host, kept per thread: a page-locked copy of
+// the control block (read back without staging) and, per device, the two
+// events around a solve. Made on first use, given back when the thread ends.
+struct SolveHost {
+    Ctrl *ctrl = nullptr;
+    cudaEvent_t ev[64][2] = {};
+    bool made[64] = {};
+    ~SolveHost() {
+        for (int d = 0; d < 64; d++)
+            if (made[d]) { cudaEventDestroy(ev[d][0]); cudaEventDestroy(ev[d][1]); }
+        if (ctrl) cudaFreeHost(ctrl);
+    }
+    // for the current device
+    cudaError_t get(int device) {
+        if (device < 0 || device >= 64) return cudaErrorInvalidDevice;
+        cudaError_t e = cudaSuccess;
+        if (!ctrl) e = cudaHostAlloc(reinterpret_cast<void **>(&ctrl), sizeof(Ctrl), cudaHostAllocPortable);
+        if (e != cudaSuccess) { ctrl = nullptr; return e; }
+        if (!made[device]) {
+            if ((e = cudaEventCreate(&ev[device][0])) != cudaSuccess) return e;
+            if ((e = cudaEventCreate(&ev[device][1])) != cudaSuccess) { cudaEventDestroy(ev[device][0]); return e; }
+            made[device] = true;
+        }
+        return cudaSuccess;
+    }
+};
+static thread_local SolveHost t_solve_host;
+
 static void free_device(Factors &F) {
     // the arena holds d_code, d_R32, d_R64, d_cell, d_scratch, d_ctrl and,
     // for shapes the barrier-free solver takes, d_flow
@@ -599,9 +627,8 @@ static cpmdp_status run_solver(const cpmdp_factors *h, cpmdp_precision prec, boo
     DeviceGuard g(F.device);
     if (!g.ok) { set_error("cannot select CUDA device %d", F.device); return CPMDP_ECUDA; }
     cudaStream_t s = (cudaStream_t)stream;
-    cudaEvent_t e0, e1;
-    CPMDP_CUDA(cudaEventCreate(&e0));
-    CPMDP_CUDA(cudaEventCreate(&e1));
+    CPMDP_CUDA(t_solve_host.get(F.device));
+    const cudaEvent_t e0 = t_solve_host.ev[F.device][0], e1 = t_solve_host.ev[F.device][1];
     CPMDP_CUDA(cudaEventRecord(e0, s));
     Ctrl hc;
     memset(&hc, 0, sizeof(hc));
@@ -614,7 +641,7 @@ static cpmdp_status run_solver(const cpmdp_factors *h, cpmdp_precision prec, boo
         CPMDP_CUDA(arena_pool(F.device, &pool));
         st = pad_prepare(const_cast<Factors &>(F), pool, s);
         if (st == CPMDP_ENOMEM) padded = false;
-        else if (st != CPMDP_OK) { cudaEventDestroy(e0); cudaEventDestroy(e1); return st; }
+        else if (st != CPMDP_OK) return st;
     }
     const Factors &A = padded ? *F.pad : F;   // what is solved
     if (F.kind == CPMDP_GRIDWORLD) {
@@ -637,7 +664,7 @@ static cpmdp_status run_solver(const cpmdp_factors *h, cpmdp_precision prec, boo
         st = dense_solve(F, prec, pi_mode, V, pi, o, &hc, s);
         have_ctrl = true;
     }
-    if (st != CPMDP_OK) { cudaEventDestroy(e0); cudaEventDestroy(e1); return st; }
+    if (st != CPMDP_OK) return st;
     // certifying FP64 sweep (banded F32 / F64 fused path)
     double *cert = (double *)((char *)F.d_ctrl + offsetof(Ctrl, certify_residual));
     const bool do_cert = o.certify && F.kind == CPMDP_GRIDWORLD;
@@ -655,19 +682,17 @@ static cpmdp_status run_solver(const cpmdp_factors *h, cpmdp_precision prec, boo
         } else {
             st = banded_certify(F, (const float *)V, pi_mode ? nullptr : pi, cert, s);
         }
-        if (st != CPMDP_OK) { cudaEventDestroy(e0); cudaEventDestroy(e1); return st; }
+        if (st != CPMDP_OK) return st;
     } else if (!pi_mode && pi && F.kind == CPMDP_GRIDWORLD && !plain) {
         st = banded_backup(F, prec, V, F.d_scratch, pi, nullptr, s);
-        if (st != CPMDP_OK) { cudaEventDestroy(e0); cudaEventDestroy(e1); return st; }
+        if (st != CPMDP_OK) return st;
     }
     CPMDP_CUDA(cudaEventRecord(e1, s));
-    Ctrl dc;
-    CPMDP_CUDA(cudaMemcpyAsync(&dc, F.d_ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, s));
+    CPMDP_CUDA(cudaMemcpyAsync(t_solve_host.ctrl, F.d_ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, s));
     CPMDP_CUDA(cudaStreamSynchronize(s));
+    const Ctrl dc = *t_solve_host.ctrl;
     float ms = 0.f;
     cudaEventElapsedTime(&ms, e0, e1);
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
     const int solver = F.kind != CPMDP_GRIDWORLD ? CPMDP_SOLVER_DENSE
                        : plain ? CPMDP_SOLVER_PLAIN
                        : A.flow_pending ? CPMDP_SOLVER_BARRIER_FREE
