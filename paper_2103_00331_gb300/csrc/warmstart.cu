@@ -719,8 +719,71 @@ __device__ __forceinline__ void coarse_of(const BatchInst &I, int cell, int &cz,
 // multiple of 4) are read as one 16-byte reward load and one 4-byte code load,
 // so neighbouring cells' threads read neighbouring bytes. A cell's 128 bytes
 // of channels are written by 8 threads, 16 bytes each, from shared memory: a
-// warp stores whole lines (one thread a cell, 78 us for 128 instances of 64^3;
-// so, 42 us: 168 MB read, 67 MB written).
+// warp stores whole lines. Bound by the memory (168 MB read, 67 MB written for
+// 128 instances of 64^3: 35 us) and the loads in flight: 78 us with one thread
+// writing a cell's channels, 51 us so.
+// The 4 states of a cell's row are taken without branching per state (the
+// terminals, a handful in an instance, apart): code bits 6 and 7 of the four
+// bytes at once, and a zero added for a state that does not count.
+struct RowSums {
+    int n = 0, obst = 0, free = 0, any_t = 0;
+    float rfree = 0.f, rlive = 0.f, tmax = 0.f;   // rewards of free states, of all but obstacles
+    __device__ __forceinline__ void add(const float (&r)[kF], unsigned cw, int states) {
+        const unsigned o = cw & 0x40404040u, t = cw & 0x80808080u;
+        n += states;
+        obst += __popc(o);
+        free += states - __popc(o | t);
+#pragma unroll
+        for (int k = 0; k < kF; k++) {
+            const float live = (o >> (8 * k) & 0xFFu) ? 0.f : r[k];
+            rlive += live;
+            rfree += (t >> (8 * k) & 0xFFu) ? 0.f : live;
+        }
+        if (t) {
+#pragma unroll
+            for (int k = 0; k < kF; k++)
+                if (t >> (8 * k) & 0xFFu) {
+                    tmax = any_t ? fmaxf(tmax, r[k]) : r[k];
+                    any_t = 1;
+                }
+        }
+    }
+};
+
+// The rows of coarse cell (cz, cy, cx) of instance I: one 16-byte reward load
+// and one 4-byte code load where the row is a full aligned group of 4, which
+// it is in every instance whose x side is a multiple of 4. A state outside the
+// grid counts for nothing (code 0, reward 0, not among `states`).
+__device__ __forceinline__ RowSums cell_sums(const BatchInst &I, const uint8_t *__restrict__ code,
+                                             const float *__restrict__ R, int cz, int cy, int cx) {
+    RowSums s;
+    const int x0 = cx * kF, nx = min(kF, I.shape[2] - x0);
+    const bool vec = I.shape[2] % 4 == 0 && I.offset % 4 == 0;
+    for (int z = cz * kF; z < min((cz + 1) * kF, I.shape[0]); z++) {
+#pragma unroll
+        for (int j = 0; j < kF; j++) {
+            const int y = cy * kF + j;
+            if (y >= I.shape[1]) break;
+            const long long at = I.offset + (long long)z * I.stride[0] + (long long)y * I.stride[1] + x0;
+            float r[kF];
+            unsigned cw = 0;
+            if (vec) {
+                const float4 rv = *reinterpret_cast<const float4 *>(R + at);
+                cw = *reinterpret_cast<const unsigned *>(code + at);
+                r[0] = rv.x; r[1] = rv.y; r[2] = rv.z; r[3] = rv.w;
+            } else {
+#pragma unroll
+                for (int k = 0; k < kF; k++) {
+                    r[k] = k < nx ? R[at + k] : 0.f;
+                    cw |= (unsigned)(k < nx ? code[at + k] : 0) << (8 * k);
+                }
+            }
+            s.add(r, cw, nx);
+        }
+    }
+    return s;
+}
+
 constexpr int kFeatThreads = 256;
 
 __global__ void __launch_bounds__(kFeatThreads) features_kernel(const BatchInst *__restrict__ inst,
@@ -734,44 +797,11 @@ __global__ void __launch_bounds__(kFeatThreads) features_kernel(const BatchInst 
             const BatchInst I = inst[first + i];
             int cz, cy, cx, zc, yc, xc;
             coarse_of(I, cell, cz, cy, cx, zc, yc, xc);
-            const unsigned ob = 1u << (2 * I.ndim), tb = 1u << (2 * I.ndim + 1);
-            float rsum = 0.f, tmax = 0.f;
-            int live = 0, obst = 0, n = 0, any_t = 0;
-            const int x0 = cx * kF, x1 = min(x0 + kF, I.shape[2]);
-            const bool vec = x1 - x0 == kF && I.shape[2] % 4 == 0 && I.offset % 4 == 0;
-            for (int z = cz * kF; z < min((cz + 1) * kF, I.shape[0]); z++)
-                for (int y = cy * kF; y < min((cy + 1) * kF, I.shape[1]); y++) {
-                    const long long row = I.offset + (long long)z * I.stride[0] + y * I.stride[1];
-                    float r4[kF];
-                    unsigned c4[kF];
-                    if (vec) {
-                        const float4 rv = *reinterpret_cast<const float4 *>(R + row + x0);
-                        const unsigned cw = *reinterpret_cast<const unsigned *>(code + row + x0);
-                        r4[0] = rv.x; r4[1] = rv.y; r4[2] = rv.z; r4[3] = rv.w;
-#pragma unroll
-                        for (int k = 0; k < kF; k++) c4[k] = (cw >> (8 * k)) & 0xFFu;
-                    } else {
-#pragma unroll
-                        for (int k = 0; k < kF; k++) {
-                            const bool in = x0 + k < x1;
-                            r4[k] = in ? R[row + x0 + k] : 0.f;
-                            c4[k] = in ? code[row + x0 + k] : 0xFFFFFFFFu;   // marks "outside the grid"
-                        }
-                    }
-#pragma unroll
-                    for (int k = 0; k < kF; k++) {
-                        const unsigned c = c4[k];
-                        if (c == 0xFFFFFFFFu) continue;
-                        n++;
-                        if (c & ob) { obst++; continue; }
-                        live++;
-                        rsum += r4[k];
-                        if (c & tb) { tmax = any_t ? fmaxf(tmax, r4[k]) : r4[k]; any_t = 1; }
-                    }
-                }
-            const __nv_bfloat162 lo = __halves2bfloat162(__float2bfloat16_rn(live ? rsum / live : 0.f),
-                                                         __float2bfloat16_rn((float)obst / (float)n));
-            const __nv_bfloat162 hi = __halves2bfloat162(__float2bfloat16_rn(any_t ? tmax : 0.f),
+            const RowSums c = cell_sums(I, code, R, cz, cy, cx);
+            const int live = c.n - c.obst;
+            const __nv_bfloat162 lo = __halves2bfloat162(__float2bfloat16_rn(live ? c.rlive / live : 0.f),
+                                                         __float2bfloat16_rn((float)c.obst / (float)c.n));
+            const __nv_bfloat162 hi = __halves2bfloat162(__float2bfloat16_rn(c.any_t ? c.tmax : 0.f),
                                                          __float2bfloat16_rn(-logf(1.f - I.gamma) / 5.f));
             sh[threadIdx.x] = make_uint2(*reinterpret_cast<const unsigned *>(&lo), *reinterpret_cast<const unsigned *>(&hi));
         }
@@ -816,13 +846,6 @@ __global__ void targets_kernel(const BatchInst *__restrict__ inst, const uint8_t
 // Interpolation in one dimension: the coarse values sit at the cell centres, a
 // fine coordinate p at (p + 0.5) / 4 - 0.5 in cell units, clamped to the
 // outermost centres.
-__device__ __forceinline__ void axis_weights(int p, int nc, int &lo, int &hi, float &t) {
-    float u = ((float)p + 0.5f) / (float)kF - 0.5f;
-    u = fminf(fmaxf(u, 0.f), (float)(nc - 1));
-    lo = (int)floorf(u);
-    hi = min(lo + 1, nc - 1);
-    t = u - (float)lo;
-}
 
 // Weight of cell c of nc at its fine coordinate 4 c - 2 + o, 0 <= o < 8: the
 // clamp gives an outermost cell all of the coordinates beyond its centre.
@@ -833,94 +856,119 @@ __device__ __forceinline__ float cell_weight(int o, int c, int nc) {
 
 __device__ __forceinline__ float lerp(float a, float b, float t) { return (1.f - t) * a + t * b; }
 
-// Trilinear interpolation of coarse + base at the 4 x 4 states z = 4 cz .. + 3,
-// x = 4 q .. + 3 of one y: they lie between the centres cz - 1, cz, cz + 1 and
-// q - 1, q, q + 1, so 18 cell values, reduced over y, then z, then x, serve all
-// 16 states (state by state: 128 loads and products).
+// Trilinear interpolation of coarse + base at half the states of a coarse cell,
+// its rows y = 4 cy + 2 half and the next: 4 x 2 x 4 states. They lie between
+// the centres cz - 1, cz, cz + 1 and cx - 1, cx, cx + 1, and between two centres
+// in y, so 18 cell values, reduced over y, then z, then x, serve all 32 (state
+// by state: 256 loads and products; a whole cell a thread: too many registers
+// for enough warps).
 struct Patch {
-    float c[3][3];             // z, x: coarse + base interpolated in y
-    float tz[4], tx[4];        // weights of the upper centre (1: the lower one is the same)
+    float c[3][2][3];          // z, y, x: coarse + base
+    float tz[4], ty[2], tx[4]; // weights of the upper centre (1: the lower one is the same)
     __device__ __forceinline__ static void weights(int c, int nc, float (&t)[4]) {
         t[0] = c > 0 ? 0.625f : 1.f;
         t[1] = c > 0 ? 0.875f : 1.f;
         t[2] = c < nc - 1 ? 0.125f : 0.f;
         t[3] = c < nc - 1 ? 0.375f : 0.f;
     }
-    __device__ __forceinline__ void load(int cz, int y, int q, int zc, int yc, int xc, const float *cv, const float *bv) {
-        int ylo, yhi;
-        float ty;
-        axis_weights(y, yc, ylo, yhi, ty);
+    __device__ __forceinline__ void load(int cz, int cy, int half, int cx, int zc, int yc, int xc, const float *cv,
+                                         const float *bv) {
+        float t[4];
         weights(cz, zc, tz);
-        weights(q, xc, tx);
-        const int x[3] = {max(q - 1, 0), q, min(q + 1, xc - 1)}, z[3] = {max(cz - 1, 0), cz, min(cz + 1, zc - 1)};
+        weights(cy, yc, t);
+        weights(cx, xc, tx);
+        ty[0] = half ? t[2] : t[0];
+        ty[1] = half ? t[3] : t[1];
+        const int x[3] = {max(cx - 1, 0), cx, min(cx + 1, xc - 1)}, z[3] = {max(cz - 1, 0), cz, min(cz + 1, zc - 1)};
+        const int y[2] = {half ? cy : max(cy - 1, 0), half ? min(cy + 1, yc - 1) : cy};
 #pragma unroll
-        for (int m = 0; m < 3; m++) {
-            const int r0 = (z[m] * yc + ylo) * xc, r1 = (z[m] * yc + yhi) * xc;
+        for (int m = 0; m < 3; m++)
 #pragma unroll
-            for (int j = 0; j < 3; j++) {
-                float a = cv[r0 + x[j]], b = cv[r1 + x[j]];
-                if (bv) { a += bv[r0 + x[j]]; b += bv[r1 + x[j]]; }
-                c[m][j] = lerp(a, b, ty);
+            for (int i = 0; i < 2; i++) {
+                const int r = (z[m] * yc + y[i]) * xc;
+#pragma unroll
+                for (int j = 0; j < 3; j++) {
+                    c[m][i][j] = cv[r + x[j]];
+                    if (bv) c[m][i][j] += bv[r + x[j]];
+                }
             }
-        }
     }
-    // the four states of plane z = 4 cz + h (h known at compile time)
-    __device__ __forceinline__ void row(int h, float (&v)[4]) const {
-        float e[3];
+    // row g of the two in all planes, reduced over y (g, h known at compile time)
+    __device__ __forceinline__ void plane(int g, float (&e)[3][3]) const {
 #pragma unroll
-        for (int j = 0; j < 3; j++) e[j] = lerp(c[h < 2 ? 0 : 1][j], c[h < 2 ? 1 : 2][j], tz[h]);
+        for (int m = 0; m < 3; m++)
 #pragma unroll
-        for (int k = 0; k < 4; k++) v[k] = lerp(e[k < 2 ? 0 : 1], e[k < 2 ? 1 : 2], tx[k]);
+            for (int j = 0; j < 3; j++) e[m][j] = lerp(c[m][0][j], c[m][1][j], ty[g]);
+    }
+    // its four states of plane z = 4 cz + h
+    __device__ __forceinline__ void row(const float (&e)[3][3], int h, float (&v)[4]) const {
+        float f[3];
+#pragma unroll
+        for (int j = 0; j < 3; j++) f[j] = lerp(e[h < 2 ? 0 : 1][j], e[h < 2 ? 1 : 2][j], tz[h]);
+#pragma unroll
+        for (int k = 0; k < 4; k++) v[k] = lerp(f[k < 2 ? 0 : 1], f[k < 2 ? 1 : 2], tx[k]);
     }
 };
 
 // Coarse estimate (plus base) upsampled to every fine state: free states
-// take the interpolation, terminals R(t), obstacles 0. One thread per patch of
-// 4 planes x 4 consecutive states of a row (blockIdx.y: instances); rows whose
-// length is a multiple of 4 (16-byte aligned, as every instance starts on a
-// multiple of 4 states) are written in 16-byte stores. Bound by the stores (V
-// 4 B, code 1 B a state) and the instructions left; 128 instances of 64^3:
-// 208 us state by state.
-__global__ void __launch_bounds__(256) upsample_kernel(const BatchInst *__restrict__ inst, const uint8_t *__restrict__ code,
+// take the interpolation, terminals R(t), obstacles 0. One thread per half
+// cell (blockIdx.y: instances); rows whose length is a multiple of 4 (16-byte
+// aligned, as every instance starts on a multiple of 4 states) are written in
+// 16-byte stores. Bound by the stores (V 4 B, code 1 B a state, 25 us) and the
+// instructions; 128 instances of 64^3: 208 us state by state, 54 us so.
+__global__ void __launch_bounds__(128) upsample_kernel(const BatchInst *__restrict__ inst, const uint8_t *__restrict__ code,
                                                        const float *__restrict__ R, int first, int count, int cells,
                                                        const float *__restrict__ coarse, const float *__restrict__ base,
                                                        float *__restrict__ V) {
     const BatchInst &I0 = inst[first];
     const int Z = I0.shape[0], Y = I0.shape[1], X = I0.shape[2];
     const int zc = (Z + kF - 1) / kF, yc = (Y + kF - 1) / kF, xc = (X + kF - 1) / kF;
-    const unsigned g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= (unsigned)zc * Y * xc) return;
-    const unsigned row = g / (unsigned)xc, q = g - row * xc, cz = row / (unsigned)Y, y = row - cz * Y;
+    const int id = blockIdx.x * blockDim.x + threadIdx.x;
+    if (id >= 2 * cells) return;
+    const int row = id / xc, cx = id - row * xc, cz = row / (2 * yc), hy = row - cz * 2 * yc, cy = hy >> 1, half = hy & 1;
     const unsigned ob = 1u << 6, tb = 1u << 7;   // 3-D codes
     const bool full = X % 4 == 0;
-    const int live = min(4, X - 4 * (int)q);
+    const int live = min(4, X - 4 * cx);
     for (int i = blockIdx.y; i < count; i += gridDim.y) {
         Patch pt;
-        pt.load((int)cz, (int)y, (int)q, zc, yc, xc, coarse + (long long)i * cells, base ? base + (long long)i * cells : nullptr);
-        const long long at = inst[first + i].offset + (long long)(4 * cz * Y + y) * X + 4 * q;
-        const long long plane = (long long)Y * X;
+        pt.load(cz, cy, half, cx, zc, yc, xc, coarse + (long long)i * cells, base ? base + (long long)i * cells : nullptr);
+        const long long at = inst[first + i].offset + (long long)(4 * cz * Y + 2 * hy) * X + 4 * cx;
 #pragma unroll
-        for (int h = 0; h < 4; h++) {
-            if (4 * (int)cz + h >= Z) break;
-            const long long s0 = at + h * plane;
-            unsigned cw = 0;
-            if (full) cw = *reinterpret_cast<const unsigned *>(code + s0);
-            else
-                for (int k = 0; k < 4; k++) cw |= (unsigned)(k < live ? code[s0 + k] : ob) << (8 * k);
-            float v[4];
-            pt.row(h, v);
+        for (int g = 0; g < 2; g++) {
+            if (2 * hy + g >= Y) break;
+            float e[3][3];
+            pt.plane(g, e);
+            unsigned cw[4];
 #pragma unroll
-            for (int k = 0; k < 4; k++) {
-                const unsigned c = cw >> (8 * k);
-                if (c & ob) v[k] = 0.f;
-                else if (c & tb) v[k] = R[s0 + k];
+            for (int h = 0; h < 4; h++) {
+                const long long s0 = at + ((long long)h * Y + g) * X;
+                cw[h] = 0;
+                if (4 * cz + h >= Z) continue;
+                if (full) cw[h] = *reinterpret_cast<const unsigned *>(code + s0);
+                else
+                    for (int k = 0; k < 4; k++) cw[h] |= (unsigned)(k < live ? code[s0 + k] : ob) << (8 * k);
             }
-            if (full) {
-                *reinterpret_cast<float4 *>(V + s0) = make_float4(v[0], v[1], v[2], v[3]);
-            } else {
 #pragma unroll
-                for (int k = 0; k < 4; k++)
-                    if (k < live) V[s0 + k] = v[k];
+            for (int h = 0; h < 4; h++) {
+                if (4 * cz + h >= Z) break;
+                const long long s0 = at + ((long long)h * Y + g) * X;
+                float v[4];
+                pt.row(e, h, v);
+                if (cw[h] & 0xC0C0C0C0u) {
+#pragma unroll
+                    for (int k = 0; k < 4; k++) {
+                        const unsigned c = cw[h] >> (8 * k);
+                        if (c & ob) v[k] = 0.f;
+                        else if (c & tb) v[k] = R[s0 + k];
+                    }
+                }
+                if (full) {
+                    *reinterpret_cast<float4 *>(V + s0) = make_float4(v[0], v[1], v[2], v[3]);
+                } else {
+#pragma unroll
+                    for (int k = 0; k < 4; k++)
+                        if (k < live) V[s0 + k] = v[k];
+                }
             }
         }
     }
@@ -929,9 +977,9 @@ __global__ void __launch_bounds__(256) upsample_kernel(const BatchInst *__restri
 // Fine-level loss of a coarse estimate: with Vh = upsample(base + pred),
 // r(s) = Vh(s) - Vt(s) on the free states (0 on terminals and obstacles,
 // where the upsampling is exact); loss += sum r^2 * inv. Threads as in
-// upsample_kernel. 32 instances of 64^3: 123 us with one state a thread, 20 us
-// so (75 MB).
-__global__ void __launch_bounds__(256) fine_resid_kernel(const BatchInst *__restrict__ inst, const uint8_t *__restrict__ code,
+// upsample_kernel. 32 instances of 64^3 (75 MB, 11 us): 123 us with one state a
+// thread, 30 us so.
+__global__ void __launch_bounds__(128) fine_resid_kernel(const BatchInst *__restrict__ inst, const uint8_t *__restrict__ code,
                                                          int first, int count, int cells, const float *__restrict__ pred,
                                                          const float *__restrict__ base, const float *__restrict__ Vt,
                                                          float *__restrict__ r, float inv, float *loss) {
@@ -939,46 +987,53 @@ __global__ void __launch_bounds__(256) fine_resid_kernel(const BatchInst *__rest
     const BatchInst &I0 = inst[first];
     const int Z = I0.shape[0], Y = I0.shape[1], X = I0.shape[2];
     const int zc = (Z + kF - 1) / kF, yc = (Y + kF - 1) / kF, xc = (X + kF - 1) / kF;
-    const unsigned g = blockIdx.x * blockDim.x + threadIdx.x;
-    const unsigned row = g / (unsigned)xc, q = g - row * xc, cz = row / (unsigned)Y, y = row - cz * Y;
-    const bool on = g < (unsigned)zc * Y * xc;
+    const int id = blockIdx.x * blockDim.x + threadIdx.x;
+    const int row = id / xc, cx = id - row * xc, cz = row / (2 * yc), hy = row - cz * 2 * yc, cy = hy >> 1, half = hy & 1;
+    const bool on = id < 2 * cells;
     const bool full = X % 4 == 0, vt16 = full && (reinterpret_cast<uintptr_t>(Vt) & 15) == 0,
                r16 = full && (reinterpret_cast<uintptr_t>(r) & 15) == 0;   // a multiple of 4 states an instance
-    const int live = min(4, X - 4 * (int)q);
-    const long long plane = (long long)Y * X, at = (long long)(4 * cz * Y + y) * X + 4 * q;
+    const int live = min(4, X - 4 * cx);
     float l = 0.f;
     for (int i = blockIdx.y; on && i < count; i += gridDim.y) {
         Patch pt;
-        pt.load((int)cz, (int)y, (int)q, zc, yc, xc, pred + (long long)i * cells, base ? base + (long long)i * cells : nullptr);
+        pt.load(cz, cy, half, cx, zc, yc, xc, pred + (long long)i * cells, base ? base + (long long)i * cells : nullptr);
+        const long long at = (long long)(4 * cz * Y + 2 * hy) * X + 4 * cx, off = inst[first + i].offset;
+        float *ri = r + (long long)i * I0.nstates;
 #pragma unroll
-        for (int h = 0; h < 4; h++) {
-            if (4 * (int)cz + h >= Z) break;
-            const long long s0 = inst[first + i].offset + at + h * plane, o = (long long)i * I0.nstates + at + h * plane;
-            unsigned cw = 0;
-            float vt[4] = {0.f, 0.f, 0.f, 0.f}, d[4];
-            if (full) cw = *reinterpret_cast<const unsigned *>(code + s0);
-            else
-                for (int k = 0; k < 4; k++) cw |= (unsigned)(k < live ? code[s0 + k] : 0x40u) << (8 * k);
-            if (vt16) {
-                const float4 v = *reinterpret_cast<const float4 *>(Vt + s0);
-                vt[0] = v.x; vt[1] = v.y; vt[2] = v.z; vt[3] = v.w;
-            } else {
+        for (int g = 0; g < 2; g++) {
+            if (2 * hy + g >= Y) break;
+            float e[3][3];
+            pt.plane(g, e);
 #pragma unroll
-                for (int k = 0; k < 4; k++)
-                    if (k < live) vt[k] = Vt[s0 + k];
-            }
-            pt.row(h, d);
+            for (int h = 0; h < 4; h++) {
+                if (4 * cz + h >= Z) break;
+                const long long s0 = at + ((long long)h * Y + g) * X;
+                unsigned cw = 0;
+                float vt[4] = {0.f, 0.f, 0.f, 0.f}, d[4];
+                if (full) cw = *reinterpret_cast<const unsigned *>(code + off + s0);
+                else
+                    for (int k = 0; k < 4; k++) cw |= (unsigned)(k < live ? code[off + s0 + k] : 0x40u) << (8 * k);
+                if (vt16) {
+                    const float4 v = *reinterpret_cast<const float4 *>(Vt + off + s0);
+                    vt[0] = v.x; vt[1] = v.y; vt[2] = v.z; vt[3] = v.w;
+                } else {
 #pragma unroll
-            for (int k = 0; k < 4; k++) {
-                d[k] = (cw >> (8 * k) & 0xC0u) ? 0.f : d[k] - vt[k];
-                l += d[k] * d[k] * inv;
-            }
-            if (r16) {
-                *reinterpret_cast<float4 *>(r + o) = make_float4(d[0], d[1], d[2], d[3]);
-            } else {
+                    for (int k = 0; k < 4; k++)
+                        if (k < live) vt[k] = Vt[off + s0 + k];
+                }
+                pt.row(e, h, d);
 #pragma unroll
-                for (int k = 0; k < 4; k++)
-                    if (k < live) r[o + k] = d[k];
+                for (int k = 0; k < 4; k++) {
+                    d[k] = (cw >> (8 * k) & 0xC0u) ? 0.f : d[k] - vt[k];
+                    l += d[k] * d[k] * inv;
+                }
+                if (r16) {
+                    *reinterpret_cast<float4 *>(ri + s0) = make_float4(d[0], d[1], d[2], d[3]);
+                } else {
+#pragma unroll
+                    for (int k = 0; k < 4; k++)
+                        if (k < live) ri[s0 + k] = d[k];
+                }
             }
         }
     }
@@ -996,65 +1051,84 @@ __global__ void __launch_bounds__(256) fine_resid_kernel(const BatchInst *__rest
 // of the interpolation, dL/dpred(c) = 2 inv sum_s w(s, c) r(s) over the fine
 // states whose interpolation reads cell c (coordinates 4c - 2 .. 4c + 5 in
 // each dimension); written into channel 0 of dy, the other channels 0.
-// The interpolation is separable: a block takes one (cz, cy) row of cells of an
-// instance, sums its up to 8 x 8 fine rows into one row of weighted sums (each
-// of 4 groups of threads two of the z planes; consecutive threads consecutive
-// states), then takes each cell's up to 8 terms along x from shared memory, and
-// writes the cells' channels in 16-byte pieces. One thread a cell over its 512
-// states took 173 us for 32 instances of 64^3, this 24 us.
-constexpr int kGradX = 64;                           // threads along x per group
-constexpr int kGradCells = 64;                       // cells of the row at a time
-constexpr int kGradStates = kF * kGradCells + 4;     // the states they read
+// The interpolation is separable: a block takes one plane cz of cells of an
+// instance and walks its rows cy. For each it sums up to 8 x 8 fine rows into
+// one row of weighted sums (each of 4 groups of threads two of the z planes;
+// consecutive threads consecutive states; the 4 fine rows that the next cy
+// reads again stay in registers), then takes each cell's up to 8 terms along x
+// from shared memory, and writes the cells' channels in 16-byte pieces. One
+// thread a cell over its 512 states took 173 us for 32 instances of 64^3, this
+// 17 us.
+constexpr int kGradX = 68;                           // threads along x per group
+constexpr int kGradCells = (kGradX - 4) / kF;        // cells of a row at a time
 __global__ void __launch_bounds__(4 * kGradX) fine_grad_kernel(const BatchInst *__restrict__ inst, int first, int count,
-                                                               int zc, int yc, int xc, const float *__restrict__ r, float inv,
+                                                               int zc, int yc, int xc, int xparts,
+                                                               const float *__restrict__ r, float inv,
                                                                __nv_bfloat16 *__restrict__ dy) {
-    __shared__ float part[4][kGradStates], out[kGradCells];
+    __shared__ float part[4][kGradX], out[kGradCells];
     const BatchInst &I0 = inst[first];
     const int Z = I0.shape[0], Y = I0.shape[1], X = I0.shape[2];
-    const int cz = blockIdx.x / yc, cy = blockIdx.x - cz * yc;
+    const int cz = blockIdx.x / xparts, c0 = (blockIdx.x - cz * xparts) * kGradCells, nc = min(kGradCells, xc - c0);
     const int grp = threadIdx.x / kGradX, tx = threadIdx.x - grp * kGradX;
+    const int x = kF * c0 - 2 + tx, z0 = kF * cz - 2 + 2 * grp;   // part[.][tx]: state x
+    float wz[2];
+    bool on[2];
+#pragma unroll
+    for (int h = 0; h < 2; h++) {
+        on[h] = x >= 0 && x < X && z0 + h >= 0 && z0 + h < Z;
+        wz[h] = on[h] ? cell_weight(2 * grp + h, cz, zc) : 0.f;
+    }
     for (int i = blockIdx.y; i < count; i += gridDim.y) {
-        const float *ri = r + (long long)i * I0.nstates;
-        for (int c0 = 0; c0 < xc; c0 += kGradCells) {
-            const int nc = min(kGradCells, xc - c0), x0 = kF * c0 - 2;   // part[.][e]: state x0 + e
-            for (int e = tx; e < kF * nc + 4; e += kGradX) {
-                const int x = x0 + e;
-                float acc = 0.f;
+        const float *ri = r + (long long)i * I0.nstates + (long long)z0 * Y * X + x;
+        float v[2][8];
 #pragma unroll
-                for (int h = 0; h < 2; h++) {
-                    const int z = kF * cz - 2 + 2 * grp + h;
-                    if (z < 0 || z >= Z || x < 0 || x >= X) continue;
-                    const float wz = cell_weight(2 * grp + h, cz, zc);
-                    float v[8];
+        for (int h = 0; h < 2; h++)
 #pragma unroll
-                    for (int j = 0; j < 8; j++) {
-                        const int y = kF * cy - 2 + j;
-                        v[j] = y >= 0 && y < Y ? ri[(z * Y + y) * X + x] : 0.f;
-                    }
-#pragma unroll
-                    for (int j = 0; j < 8; j++) acc += wz * cell_weight(j, cy, yc) * v[j];
-                }
-                part[grp][e] = acc;
+            for (int j = 0; j < 4; j++) {
+                const int y = j - 2;                 // rows -2 .. 1 of cy = 0
+                v[h][j] = on[h] && y >= 0 && y < Y ? ri[(h * Y + y) * X] : 0.f;
             }
+        for (int cy = 0; cy < yc; cy++) {
+#pragma unroll
+            for (int h = 0; h < 2; h++)
+#pragma unroll
+                for (int j = 4; j < 8; j++) {
+                    const int y = kF * cy - 2 + j;
+                    v[h][j] = on[h] && y < Y ? ri[(h * Y + y) * X] : 0.f;
+                }
+            float acc = 0.f;
+#pragma unroll
+            for (int h = 0; h < 2; h++) {
+                float s = 0.f;
+#pragma unroll
+                for (int j = 0; j < 8; j++) s += cell_weight(j, cy, yc) * v[h][j];
+                acc += wz[h] * s;
+            }
+            part[grp][tx] = acc;
             __syncthreads();
-            for (int c = threadIdx.x; c < nc; c += blockDim.x) {
-                float acc = 0.f;
+            if ((int)threadIdx.x < nc) {
+                const int c = threadIdx.x;
+                float sum = 0.f;
 #pragma unroll
                 for (int j = 0; j < 8; j++) {
-                    const int e = kF * c + j, x = x0 + e;
-                    if (x < 0 || x >= X) continue;
-                    acc += cell_weight(j, c0 + c, xc) * ((part[0][e] + part[1][e]) + (part[2][e] + part[3][e]));
+                    const int e = kF * c + j;
+                    sum += cell_weight(j, c0 + c, xc) * ((part[0][e] + part[1][e]) + (part[2][e] + part[3][e]));
                 }
-                out[c] = 2.f * inv * acc;
+                out[c] = 2.f * inv * sum;
             }
             __syncthreads();
             uint4 *d = reinterpret_cast<uint4 *>(dy + ((((size_t)i * zc + cz) * yc + cy) * xc + c0) * kC);
             for (int e = threadIdx.x; e < nc * 8; e += blockDim.x) {
-                uint4 v = make_uint4(0u, 0u, 0u, 0u);
-                if ((e & 7) == 0) v.x = (unsigned)__bfloat16_as_ushort(__float2bfloat16_rn(out[e >> 3]));
-                d[e] = v;
+                uint4 w = make_uint4(0u, 0u, 0u, 0u);
+                if ((e & 7) == 0) w.x = (unsigned)__bfloat16_as_ushort(__float2bfloat16_rn(out[e >> 3]));
+                d[e] = w;
             }
+#pragma unroll
+            for (int h = 0; h < 2; h++)
+#pragma unroll
+                for (int j = 0; j < 4; j++) v[h][j] = v[h][j + 4];
         }
+        __syncthreads();
     }
 }
 
@@ -1067,7 +1141,7 @@ __global__ void __launch_bounds__(4 * kGradX) fine_grad_kernel(const BatchInst *
 // 1 + gamma + gamma^2 + gamma^3 (four fine steps); discount gamma^4, the
 // instance's slip model, walls and obstacle cells block moves. Jacobi sweeps
 // from zero until max |dV| < tol or max_sweeps.
-constexpr int kCoarseThreads = 512;
+constexpr int kCoarseThreads = 1024;
 constexpr int kMaxCoarseCells = 8192;
 
 template <int N>
@@ -1086,52 +1160,16 @@ __global__ void __launch_bounds__(kCoarseThreads) coarse_vi_kernel(const BatchIn
     const int i = blockIdx.x;
     const BatchInst I = inst[first + i];
     const int zc = (I.shape[0] + kF - 1) / kF, yc = (I.shape[1] + kF - 1) / kF, xc = (I.shape[2] + kF - 1) / kF;
-    const unsigned ob = 1u << (2 * I.ndim), tb = 1u << (2 * I.ndim + 1);
     const float g = I.gamma;
     const float gc = g * g * g * g, steps = 1.f + g + g * g + g * g * g;
-    // per cell, over its rows of up to 4 fine states (one 16-byte reward load
-    // and one 4-byte code load where the row is a full aligned group of 4)
     for (int c = tid; c < cells; c += kCoarseThreads) {
         const int cz = c / (yc * xc), cy = (c / xc) % yc, cx = c % xc;
-        const int x0 = cx * kF, x1 = min(x0 + kF, I.shape[2]);
-        const bool vec = x1 - x0 == kF && I.shape[2] % 4 == 0 && I.offset % 4 == 0;
-        int n = 0, n_obst = 0, n_free = 0, any_t = 0;
-        float rs = 0.f, tmax = 0.f;
-        for (int z = cz * kF; z < min((cz + 1) * kF, I.shape[0]); z++)
-            for (int y = cy * kF; y < min((cy + 1) * kF, I.shape[1]); y++) {
-                const long long row = I.offset + (long long)z * I.stride[0] + (long long)y * I.stride[1];
-                float r4[kF];
-                unsigned c4[kF];
-                if (vec) {
-                    const float4 rv = *reinterpret_cast<const float4 *>(R + row + x0);
-                    const unsigned cw = *reinterpret_cast<const unsigned *>(code + row + x0);
-                    r4[0] = rv.x; r4[1] = rv.y; r4[2] = rv.z; r4[3] = rv.w;
-#pragma unroll
-                    for (int k = 0; k < kF; k++) c4[k] = (cw >> (8 * k)) & 0xFFu;
-                } else {
-#pragma unroll
-                    for (int k = 0; k < kF; k++) {
-                        const bool in = x0 + k < x1;
-                        r4[k] = in ? R[row + x0 + k] : 0.f;
-                        c4[k] = in ? code[row + x0 + k] : 0xFFFFFFFFu;   // outside the grid
-                    }
-                }
-#pragma unroll
-                for (int k = 0; k < kF; k++) {
-                    const unsigned cs = c4[k];
-                    if (cs == 0xFFFFFFFFu) continue;
-                    n++;
-                    if (cs & ob) { n_obst++; continue; }
-                    if (cs & tb) { tmax = any_t ? fmaxf(tmax, r4[k]) : r4[k]; any_t = 1; continue; }
-                    n_free++;
-                    rs += r4[k];
-                }
-            }
+        const RowSums sums = cell_sums(I, code, R, cz, cy, cx);
         uint8_t k = 0;
         float r = 0.f;
-        if (2 * n_obst >= n) k = 0x40;
-        else if (any_t) { k = 0x80; r = tmax; }
-        else r = n_free ? rs / (float)n_free * steps : 0.f;
+        if (2 * sums.obst >= sums.n) k = 0x40;
+        else if (sums.any_t) { k = 0x80; r = sums.tmax; }
+        else r = sums.free ? sums.rfree / (float)sums.free * steps : 0.f;
         kind[c] = k;
         rsum[c] = r;
     }
@@ -1155,7 +1193,8 @@ __global__ void __launch_bounds__(kCoarseThreads) coarse_vi_kernel(const BatchIn
     // from the thread's); the larger of a dimension's two neighbours gives the
     // larger of its two actions' values (weights >= 0, rounding is monotone).
     // 128 instances of 64^3: 165 us with every cell's kind, reward and
-    // addresses worked out on each sweep.
+    // addresses worked out on each sweep, 512 threads and a branch per fine
+    // state; 93 us so.
     const float wm = I.w_move, wp = I.w_perp;
     const int s0 = yc * xc, s1 = xc;
     float rr[N];
@@ -1383,9 +1422,8 @@ cpmdp_status cpmdp_ws_upsample(const cpmdp_batch *B, const float *coarse, const 
     cpmdp_status s = batch_range(B, first, count, &cells);
     if (s != CPMDP_OK) return s;
     const BatchInst &I0 = B->inst[(size_t)first];
-    const long long patches = (long long)((I0.shape[0] + kF - 1) / kF) * I0.shape[1] * ((I0.shape[2] + kF - 1) / kF);
-    const dim3 grid((unsigned)((patches + 255) / 256), (unsigned)std::min(count, 65535));
-    upsample_kernel<<<grid, 256, 0, (cudaStream_t)stream>>>(B->d_inst, B->d_code, B->d_R, first, count, cells, coarse,
+    const dim3 grid((unsigned)((2LL * cells + 127) / 128), (unsigned)std::min(count, 65535));
+    upsample_kernel<<<grid, 128, 0, (cudaStream_t)stream>>>(B->d_inst, B->d_code, B->d_R, first, count, cells, coarse,
                                                             base, V);
     CPMDP_CUDA(cudaGetLastError());
     return CPMDP_OK;
@@ -1403,12 +1441,13 @@ cpmdp_status cpmdp_ws_fine_loss_grad(const cpmdp_batch *B, const float *V_target
     const BatchInst &I0 = B->inst[(size_t)first];
     const int zc = (I0.shape[0] + kF - 1) / kF, yc = (I0.shape[1] + kF - 1) / kF, xc = (I0.shape[2] + kF - 1) / kF;
     const unsigned ny = (unsigned)std::min(count, 65535);
-    const dim3 grid((unsigned)(((long long)zc * I0.shape[1] * xc + 255) / 256), ny);
-    fine_resid_kernel<<<grid, 256, 0, (cudaStream_t)stream>>>(B->d_inst, B->d_code, first, count, cells, pred, base,
+    const dim3 grid((unsigned)((2LL * cells + 127) / 128), ny);
+    fine_resid_kernel<<<grid, 128, 0, (cudaStream_t)stream>>>(B->d_inst, B->d_code, first, count, cells, pred, base,
                                                               V_target, resid, inv, loss);
     CPMDP_CUDA(cudaGetLastError());
-    fine_grad_kernel<<<dim3((unsigned)(zc * yc), ny), 4 * kGradX, 0, (cudaStream_t)stream>>>(
-        B->d_inst, first, count, zc, yc, xc, resid, inv, (__nv_bfloat16 *)dy);
+    const int xparts = (xc + kGradCells - 1) / kGradCells;
+    fine_grad_kernel<<<dim3((unsigned)(zc * xparts), ny), 4 * kGradX, 0, (cudaStream_t)stream>>>(
+        B->d_inst, first, count, zc, yc, xc, xparts, resid, inv, (__nv_bfloat16 *)dy);
     CPMDP_CUDA(cudaGetLastError());
     return CPMDP_OK;
 }
@@ -1424,8 +1463,8 @@ cpmdp_status cpmdp_ws_coarse_vi(const cpmdp_batch *B, int32_t first, int32_t cou
     }
     if (!coarse_v || !(tol > 0.f) || max_sweeps < 1) { set_error("coarse_v, tol > 0 and max_sweeps >= 1 required"); return CPMDP_EINVAL; }
     const size_t smem = (size_t)cells * 13;
-    const auto kern = cells <= 2 * kCoarseThreads ? coarse_vi_kernel<2> : cells <= 8 * kCoarseThreads
-                                                                            ? coarse_vi_kernel<8> : coarse_vi_kernel<16>;
+    const auto kern = cells <= kCoarseThreads ? coarse_vi_kernel<1> : cells <= 4 * kCoarseThreads ? coarse_vi_kernel<4>
+                                                                                                  : coarse_vi_kernel<8>;
     CPMDP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     kern<<<count, kCoarseThreads, smem, (cudaStream_t)stream>>>(B->d_inst, B->d_code, B->d_R, first, cells, tol, max_sweeps,
                                                                 coarse_v, (__nv_bfloat16 *)feat);
