@@ -319,7 +319,7 @@ static void slab_launch(const SlabArgs<T> &a, bool last, dim3 grid, cudaStream_t
 
 template <typename T>
 cudaError_t slab_sweep(const Factors &F, const T *Vin, T *Vout, uint8_t *pi, int mode, T margin,
-                       unsigned long long *res, unsigned *chg, cudaStream_t st) {
+                       unsigned long long *res, unsigned *chg, const int *stop, cudaStream_t st) {
     constexpr bool f64 = sizeof(T) == 8;
     const DenseSlab &s = *F.slab;
     const SlabPlan &plan = f64 ? s.plan64 : s.plan32;
@@ -344,6 +344,7 @@ cudaError_t slab_sweep(const Factors &F, const T *Vin, T *Vout, uint8_t *pi, int
     a.pi = pi;
     a.res = res;
     a.changed = chg;
+    a.stop = stop;
     for (int a0 = 0; a0 < F.nactions; a0 += plan.actions) {
         a.a0 = a0;
         a.a1 = std::min(F.nactions, a0 + plan.actions);
@@ -371,8 +372,8 @@ cudaError_t slab_sweep(const Factors &F, const T *Vin, T *Vout, uint8_t *pi, int
 }
 
 template cudaError_t slab_sweep<float>(const Factors &, const float *, float *, uint8_t *, int, float,
-                                       unsigned long long *, unsigned *, cudaStream_t);
+                                       unsigned long long *, unsigned *, const int *, cudaStream_t);
 template cudaError_t slab_sweep<double>(const Factors &, const double *, double *, uint8_t *, int, double,
-                                        unsigned long long *, unsigned *, cudaStream_t);
+                                        unsigned long long *, unsigned *, const int *, cudaStream_t);
 
 }  // namespace cpmdp

@@ -128,6 +128,7 @@ struct SlabArgs {
     uint8_t *pi;
     unsigned long long *res;
     unsigned *changed;
+    const int *stop;           // nullable: the sweep does nothing when it is set
     SlabPhase p;
 };
 
@@ -620,6 +621,12 @@ __global__ void __maxnreg__(IB * CB == 64 ? 168 : 128) slab_kernel(const __grid_
     slab_load_u<T>(a, a.c0 + first, min(chmax, nchains), 0, 0, us);
     load_tile(0, min(chmax, nchains), tile);
     slab_commit();
+    if (a.stop) {
+        // read while the first copies fly; the same for every thread
+        const int stopped = *a.stop;
+        slab_wait_all();
+        if (stopped) return;
+    }
     for (int c = 0; c < nchains; c += chmax) {
         const int nch = min(chmax, nchains - c);
         // this chain's products run in `work`
@@ -779,6 +786,6 @@ const SlabPlan *slab_plan(const Factors &F, size_t elem);
 // One sweep over all chains (see dense_sweep for the modes).
 template <typename T>
 cudaError_t slab_sweep(const Factors &F, const T *Vin, T *Vout, uint8_t *pi, int mode, T margin,
-                       unsigned long long *res, unsigned *chg, cudaStream_t st);
+                       unsigned long long *res, unsigned *chg, const int *stop, cudaStream_t st);
 
 }  // namespace cpmdp
