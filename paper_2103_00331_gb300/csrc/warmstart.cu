@@ -1051,84 +1051,80 @@ __global__ void __launch_bounds__(128) fine_resid_kernel(const BatchInst *__rest
 // of the interpolation, dL/dpred(c) = 2 inv sum_s w(s, c) r(s) over the fine
 // states whose interpolation reads cell c (coordinates 4c - 2 .. 4c + 5 in
 // each dimension); written into channel 0 of dy, the other channels 0.
-// The interpolation is separable: a block takes one plane cz of cells of an
-// instance and walks its rows cy. For each it sums up to 8 x 8 fine rows into
-// one row of weighted sums (each of 4 groups of threads two of the z planes;
-// consecutive threads consecutive states; the 4 fine rows that the next cy
-// reads again stay in registers), then takes each cell's up to 8 terms along x
-// from shared memory, and writes the cells' channels in 16-byte pieces. One
-// thread a cell over its 512 states took 173 us for 32 instances of 64^3, this
-// 17 us.
-constexpr int kGradX = 68;                           // threads along x per group
-constexpr int kGradCells = (kGradX - 4) / kF;        // cells of a row at a time
-__global__ void __launch_bounds__(4 * kGradX) fine_grad_kernel(const BatchInst *__restrict__ inst, int first, int count,
-                                                               int zc, int yc, int xc, int xparts,
-                                                               const float *__restrict__ r, float inv,
-                                                               __nv_bfloat16 *__restrict__ dy) {
-    __shared__ float part[4][kGradX], out[kGradCells];
+// One thread a cell, its sum in the order z, y, x (the result is rounded to
+// bf16, where another order shows as a whole last place). A block takes 16 x 16
+// cells of one cz; the fine plane under them comes to shared memory by
+// asynchronous copies, one plane ahead of the sums, each state once, and a cell
+// reads a row's 8 states as three 16-byte pieces. Bound by those reads (192 a
+// cell). 32 instances of 64^3: 173 us with every thread reading its states from
+// global memory, 39 us so (17 us with the sums taken dimension by dimension,
+// which moved 6e-7 of the gradients by a last place of bf16).
+constexpr int kGradCells = 16;                       // cells of a tile per dimension
+constexpr int kGradRows = kF * kGradCells + 4;       // fine rows under it: 4 cy0 - 2 ..
+constexpr int kGradPitch = kF * kGradCells + 8;      // fine states of a row: 4 cx0 - 4 ..
+__global__ void __launch_bounds__(kGradCells *kGradCells) fine_grad_kernel(const BatchInst *__restrict__ inst, int first,
+                                                                          int count, int zc, int yc, int xc,
+                                                                          const float *__restrict__ r, float inv,
+                                                                          __nv_bfloat16 *__restrict__ dy) {
+    __shared__ __align__(16) float plane[2][kGradRows * kGradPitch];
     const BatchInst &I0 = inst[first];
     const int Z = I0.shape[0], Y = I0.shape[1], X = I0.shape[2];
-    const int cz = blockIdx.x / xparts, c0 = (blockIdx.x - cz * xparts) * kGradCells, nc = min(kGradCells, xc - c0);
-    const int grp = threadIdx.x / kGradX, tx = threadIdx.x - grp * kGradX;
-    const int x = kF * c0 - 2 + tx, z0 = kF * cz - 2 + 2 * grp;   // part[.][tx]: state x
-    float wz[2];
-    bool on[2];
-#pragma unroll
-    for (int h = 0; h < 2; h++) {
-        on[h] = x >= 0 && x < X && z0 + h >= 0 && z0 + h < Z;
-        wz[h] = on[h] ? cell_weight(2 * grp + h, cz, zc) : 0.f;
-    }
+    const int xt = (xc + kGradCells - 1) / kGradCells, yt = (yc + kGradCells - 1) / kGradCells;
+    const int cz = blockIdx.x / (xt * yt), rest = blockIdx.x - cz * xt * yt;
+    const int cy0 = rest / xt * kGradCells, cx0 = (rest - rest / xt * xt) * kGradCells;
+    const int lx = threadIdx.x % kGradCells, ly = threadIdx.x / kGradCells, cx = cx0 + lx, cy = cy0 + ly;
+    const int x0 = kF * cx0 - 4, y0 = kF * cy0 - 2, zlo = max(0, kF * cz - 2), zhi = min(Z - 1, kF * cz + 5);
     for (int i = blockIdx.y; i < count; i += gridDim.y) {
-        const float *ri = r + (long long)i * I0.nstates + (long long)z0 * Y * X + x;
-        float v[2][8];
-#pragma unroll
-        for (int h = 0; h < 2; h++)
-#pragma unroll
-            for (int j = 0; j < 4; j++) {
-                const int y = j - 2;                 // rows -2 .. 1 of cy = 0
-                v[h][j] = on[h] && y >= 0 && y < Y ? ri[(h * Y + y) * X] : 0.f;
+        const float *ri = r + (long long)i * I0.nstates;
+        auto fetch = [&](int z) {
+            float *p = plane[z & 1];
+            const float *src = ri + (long long)z * Y * X;
+            for (int e = threadIdx.x; e < kGradRows * kGradPitch; e += kGradCells * kGradCells) {
+                const int row = e / kGradPitch, y = y0 + row, x = x0 + e - row * kGradPitch;
+                if (y >= 0 && y < Y && x >= 0 && x < X)
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(tc::smem_u32(p + e)),
+                                 "l"(src + (long long)y * X + x)
+                                 : "memory");
+                else
+                    p[e] = 0.f;
             }
-        for (int cy = 0; cy < yc; cy++) {
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+        fetch(zlo);
+        float acc = 0.f;
+        for (int z = zlo; z <= zhi; z++) {
+            if (z < zhi) {
+                fetch(z + 1);
+                asm volatile("cp.async.wait_group 1;" ::: "memory");
+            } else {
+                asm volatile("cp.async.wait_group 0;" ::: "memory");
+            }
+            __syncthreads();                         // plane z is there, for every thread
+            const float wz = cell_weight(z - (kF * cz - 2), cz, zc);
+            const float *p = plane[z & 1] + kF * ly * kGradPitch + kF * lx;
 #pragma unroll
-            for (int h = 0; h < 2; h++)
+            for (int j = 0; j < 8; j++) {
+                const float wzy = wz * cell_weight(j, cy, yc);
+                float v[12];
 #pragma unroll
-                for (int j = 4; j < 8; j++) {
-                    const int y = kF * cy - 2 + j;
-                    v[h][j] = on[h] && y < Y ? ri[(h * Y + y) * X] : 0.f;
+                for (int q = 0; q < 3; q++) {
+                    const float4 f = *reinterpret_cast<const float4 *>(p + j * kGradPitch + 4 * q);
+                    v[4 * q] = f.x; v[4 * q + 1] = f.y; v[4 * q + 2] = f.z; v[4 * q + 3] = f.w;
                 }
-            float acc = 0.f;
 #pragma unroll
-            for (int h = 0; h < 2; h++) {
-                float s = 0.f;
-#pragma unroll
-                for (int j = 0; j < 8; j++) s += cell_weight(j, cy, yc) * v[h][j];
-                acc += wz[h] * s;
+                for (int k = 0; k < 8; k++) acc = fmaf(wzy * cell_weight(k, cx, xc), v[k + 2], acc);
             }
-            part[grp][tx] = acc;
-            __syncthreads();
-            if ((int)threadIdx.x < nc) {
-                const int c = threadIdx.x;
-                float sum = 0.f;
-#pragma unroll
-                for (int j = 0; j < 8; j++) {
-                    const int e = kF * c + j;
-                    sum += cell_weight(j, c0 + c, xc) * ((part[0][e] + part[1][e]) + (part[2][e] + part[3][e]));
-                }
-                out[c] = 2.f * inv * sum;
-            }
-            __syncthreads();
-            uint4 *d = reinterpret_cast<uint4 *>(dy + ((((size_t)i * zc + cz) * yc + cy) * xc + c0) * kC);
-            for (int e = threadIdx.x; e < nc * 8; e += blockDim.x) {
-                uint4 w = make_uint4(0u, 0u, 0u, 0u);
-                if ((e & 7) == 0) w.x = (unsigned)__bfloat16_as_ushort(__float2bfloat16_rn(out[e >> 3]));
-                d[e] = w;
-            }
-#pragma unroll
-            for (int h = 0; h < 2; h++)
-#pragma unroll
-                for (int j = 0; j < 4; j++) v[h][j] = v[h][j + 4];
+            __syncthreads();                         // and read: its buffer takes plane z + 2
         }
-        __syncthreads();
+        if (cx < xc && cy < yc) {
+            uint4 *d = reinterpret_cast<uint4 *>(dy + ((((size_t)i * zc + cz) * yc + cy) * xc + cx) * kC);
+            uint4 w = make_uint4((unsigned)__bfloat16_as_ushort(__float2bfloat16_rn(2.f * inv * acc)), 0u, 0u, 0u);
+#pragma unroll
+            for (int q = 0; q < 8; q++) {
+                d[q] = w;
+                w.x = 0u;
+            }
+        }
     }
 }
 
@@ -1161,7 +1157,9 @@ __global__ void __launch_bounds__(kCoarseThreads) coarse_vi_kernel(const BatchIn
     const BatchInst I = inst[first + i];
     const int zc = (I.shape[0] + kF - 1) / kF, yc = (I.shape[1] + kF - 1) / kF, xc = (I.shape[2] + kF - 1) / kF;
     const float g = I.gamma;
-    const float gc = g * g * g * g, steps = 1.f + g + g * g + g * g * g;
+    // gamma^4 and 1 + gamma + gamma^2 + gamma^3 (the rounding spelled out, as below)
+    const float g3 = __fmul_rn(__fmul_rn(g, g), g);
+    const float gc = __fmul_rn(g3, g), steps = __fadd_rn(__fmaf_rn(g, g, __fadd_rn(1.f, g)), g3);
     for (int c = tid; c < cells; c += kCoarseThreads) {
         const int cz = c / (yc * xc), cy = (c / xc) % yc, cx = c % xc;
         const RowSums sums = cell_sums(I, code, R, cz, cy, cx);
@@ -1221,9 +1219,10 @@ __global__ void __launch_bounds__(kCoarseThreads) coarse_vi_kernel(const BatchIn
             const float n0 = (k & 1u) ? self : zm[o], n1 = (k & 2u) ? self : zp[o], n2 = (k & 4u) ? self : ym[o];
             const float n3 = (k & 8u) ? self : yp[o], n4 = (k & 16u) ? self : p[o - 1], n5 = (k & 32u) ? self : p[o + 1];
             const float P0 = n0 + n1, P1 = n2 + n3, P2 = n4 + n5;
-            float best = wm * fmaxf(n0, n1) + wp * (P1 + P2);
-            best = fmaxf(best, wm * fmaxf(n2, n3) + wp * (P0 + P2));
-            best = fmaxf(best, wm * fmaxf(n4, n5) + wp * (P0 + P1));
+            // (the rounding spelled out: the values go on as bf16 features)
+            float best = __fmaf_rn(wm, fmaxf(n0, n1), __fmul_rn(wp, P1 + P2));
+            best = fmaxf(best, __fmaf_rn(wm, fmaxf(n2, n3), __fmul_rn(wp, P0 + P2)));
+            best = fmaxf(best, __fmaf_rn(wm, fmaxf(n4, n5), __fmul_rn(wp, P0 + P1)));
             const float v = rr[n] + gc * best;
             out[o] = v;
             open |= fabsf(v - self) >= tol;
@@ -1445,9 +1444,9 @@ cpmdp_status cpmdp_ws_fine_loss_grad(const cpmdp_batch *B, const float *V_target
     fine_resid_kernel<<<grid, 128, 0, (cudaStream_t)stream>>>(B->d_inst, B->d_code, first, count, cells, pred, base,
                                                               V_target, resid, inv, loss);
     CPMDP_CUDA(cudaGetLastError());
-    const int xparts = (xc + kGradCells - 1) / kGradCells;
-    fine_grad_kernel<<<dim3((unsigned)(zc * xparts), ny), 4 * kGradX, 0, (cudaStream_t)stream>>>(
-        B->d_inst, first, count, zc, yc, xc, xparts, resid, inv, (__nv_bfloat16 *)dy);
+    const long long tiles = (long long)zc * ((yc + kGradCells - 1) / kGradCells) * ((xc + kGradCells - 1) / kGradCells);
+    fine_grad_kernel<<<dim3((unsigned)tiles, ny), kGradCells * kGradCells, 0, (cudaStream_t)stream>>>(
+        B->d_inst, first, count, zc, yc, xc, resid, inv, (__nv_bfloat16 *)dy);
     CPMDP_CUDA(cudaGetLastError());
     return CPMDP_OK;
 }
