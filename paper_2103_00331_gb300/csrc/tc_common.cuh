@@ -187,22 +187,8 @@ __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void *src, uint32_t
                  : "memory");
 }
 
-// Tiled tensor copy global -> shared of one box of a 5-D tensor map (the
-// map is a __grid_constant__ kernel parameter), completing the box's bytes
-// on the mbarrier. Coordinates are element indices, innermost first; parts
-// of the box outside the tensor are filled with zeros. The innermost
-// coordinate times the element size must be a multiple of 16 bytes.
-__device__ __forceinline__ void tma_load_5d(uint32_t dst, const void *tmap, int c0, int c1, int c2, int c3, int c4,
-                                            uint64_t *mbar) {
-    asm volatile(
-        "cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5, "
-        "%6}], [%7];" ::"r"(dst),
-        "l"(tmap), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "r"(smem_u32(mbar))
-        : "memory");
-}
-
-// The copies and the expect below, issued by the thread whose `lead` is set in
-// code that the whole warp runs (see mma_lead).
+// The copy above, issued by the thread whose `lead` is set in code that the
+// whole warp runs (see mma_lead); the same holds for the two calls below.
 __device__ __forceinline__ void bulk_g2s_lead(bool lead, uint32_t dst, const void *src, uint32_t bytes, uint64_t *mbar) {
     asm volatile(
         "{\n.reg .pred q;\nsetp.ne.b32 q, %4, 0;\n"
@@ -210,6 +196,11 @@ __device__ __forceinline__ void bulk_g2s_lead(bool lead, uint32_t dst, const voi
         "l"(src), "r"(bytes), "r"(smem_u32(mbar)), "r"((uint32_t)lead)
         : "memory");
 }
+// Tiled tensor copy global -> shared of one box of a 5-D tensor map (the
+// map is a __grid_constant__ kernel parameter), completing the box's bytes
+// on the mbarrier. Coordinates are element indices, innermost first; parts
+// of the box outside the tensor are filled with zeros. The innermost
+// coordinate times the element size must be a multiple of 16 bytes.
 __device__ __forceinline__ void tma_load_5d_lead(bool lead, uint32_t dst, const void *tmap, int c0, int c1, int c2, int c3,
                                                  int c4, uint64_t *mbar) {
     asm volatile(
@@ -219,6 +210,7 @@ __device__ __forceinline__ void tma_load_5d_lead(bool lead, uint32_t dst, const 
         "l"(tmap), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "r"(smem_u32(mbar)), "r"((uint32_t)lead)
         : "memory");
 }
+// mbar_expect_tx (below) of the lead thread.
 __device__ __forceinline__ void mbar_expect_tx_lead(bool lead, uint64_t *mbar, uint32_t bytes) {
     asm volatile("{\n.reg .pred q;\nsetp.ne.b32 q, %2, 0;\n@q mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n}\n" ::"r"(
                      smem_u32(mbar)),

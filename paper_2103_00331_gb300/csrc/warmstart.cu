@@ -714,14 +714,6 @@ __device__ __forceinline__ void coarse_of(const BatchInst &I, int cell, int &cz,
     cz = cell / (xc * yc);
 }
 
-// One thread per coarse cell (blockIdx.y: instances); rows of the cell whose x
-// extent is a full aligned group of 4 (every row of an instance with x side a
-// multiple of 4) are read as one 16-byte reward load and one 4-byte code load,
-// so neighbouring cells' threads read neighbouring bytes. A cell's 128 bytes
-// of channels are written by 8 threads, 16 bytes each, from shared memory: a
-// warp stores whole lines. Bound by the memory (168 MB read, 67 MB written for
-// 128 instances of 64^3: 35 us) and the loads in flight: 78 us with one thread
-// writing a cell's channels, 51 us so.
 // The 4 states of a cell's row are taken without branching per state (the
 // terminals, a handful in an instance, apart): code bits 6 and 7 of the four
 // bytes at once, and a zero added for a state that does not count.
@@ -786,6 +778,14 @@ __device__ __forceinline__ RowSums cell_sums(const BatchInst &I, const uint8_t *
 
 constexpr int kFeatThreads = 256;
 
+// One thread per coarse cell (blockIdx.y: instances); rows of the cell whose x
+// extent is a full aligned group of 4 (every row of an instance with x side a
+// multiple of 4) are read as one 16-byte reward load and one 4-byte code load,
+// so neighbouring cells' threads read neighbouring bytes. A cell's 128 bytes
+// of channels are written by 8 threads, 16 bytes each, from shared memory: a
+// warp stores whole lines. Bound by the memory (168 MB read, 67 MB written for
+// 128 instances of 64^3: 35 us) and the loads in flight: 78 us with one thread
+// writing a cell's channels, 51 us so.
 __global__ void __launch_bounds__(kFeatThreads) features_kernel(const BatchInst *__restrict__ inst,
                                                                 const uint8_t *__restrict__ code,
                                                                 const float *__restrict__ R, int first, int count,
@@ -846,7 +846,6 @@ __global__ void targets_kernel(const BatchInst *__restrict__ inst, const uint8_t
 // Interpolation in one dimension: the coarse values sit at the cell centres, a
 // fine coordinate p at (p + 0.5) / 4 - 0.5 in cell units, clamped to the
 // outermost centres.
-
 // Weight of cell c of nc at its fine coordinate 4 c - 2 + o, 0 <= o < 8: the
 // clamp gives an outermost cell all of the coordinates beyond its centre.
 __device__ __forceinline__ float cell_weight(int o, int c, int nc) {
