@@ -135,7 +135,9 @@ typedef struct {
                                 (at most 256 segments of the vector width) run in a single block with
                                 the values in shared memory (same values and sweep counts as the
                                 grid-barrier solver); FP32 GridWorld solves of
-                                1 to 3 dimensions whose rows are a multiple of 4 states and that fit
+                                1 to 3 dimensions whose rows are a multiple of 4 states (other rows:
+                                on a copy with the rows padded to it, where that adds at most a
+                                third and the memory is there) and that fit
                                 one co-resident grid at one thread per column of 1, 2 or 4 segments of
                                 4 states run barrier-free (sweeps synchronised through sweep-tagged
                                 values, the stopping rule checked three sweeps late; same values and
@@ -204,7 +206,10 @@ void cpmdp_default_opts(cpmdp_solve_opts *opts);
  * factors, plus the obstacle and terminal correction, encoded per state;
  * dense -> the given factors. Copies rewards, codes and factors to device
  * `device` and allocates the solvers' scratch there (about 8 bytes per
- * state; dense adds 2 value tensors). device = -1 builds a host-only object
+ * state; dense adds 2 value tensors and the intermediates of its fused
+ * sweeps, whole actions of them up to 1 GiB and at least one action).
+ * FP32 solves of rows that are no multiple of 4 states add a padded copy of
+ * the model when first called. device = -1 builds a host-only object
  * usable by cpmdp_factors_info and cpmdp_components only.
  * On success *out owns everything; release it with cpmdp_free_factors.
  * Errors: EINVAL (problem invalid), ENOMEM, ECUDA.
