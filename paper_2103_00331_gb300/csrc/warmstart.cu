@@ -1058,6 +1058,7 @@ __global__ void __launch_bounds__(128) fine_resid_kernel(const BatchInst *__rest
 // cell). 32 instances of 64^3: 173 us with every thread reading its states from
 // global memory, 39 us so (17 us with the sums taken dimension by dimension,
 // which moved 6e-7 of the gradients by a last place of bf16).
+// A cell's channels are written in 16-byte stores where dy lies so, else one by one.
 constexpr int kGradCells = 16;                       // cells of a tile per dimension
 constexpr int kGradRows = kF * kGradCells + 4;       // fine rows under it: 4 cy0 - 2 ..
 constexpr int kGradPitch = kF * kGradCells + 8;      // fine states of a row: 4 cx0 - 4 ..
@@ -1116,12 +1117,19 @@ __global__ void __launch_bounds__(kGradCells *kGradCells) fine_grad_kernel(const
             __syncthreads();                         // and read: its buffer takes plane z + 2
         }
         if (cx < xc && cy < yc) {
-            uint4 *d = reinterpret_cast<uint4 *>(dy + ((((size_t)i * zc + cz) * yc + cy) * xc + cx) * kC);
-            uint4 w = make_uint4((unsigned)__bfloat16_as_ushort(__float2bfloat16_rn(2.f * inv * acc)), 0u, 0u, 0u);
+            __nv_bfloat16 *d = dy + ((((size_t)i * zc + cz) * yc + cy) * xc + cx) * kC;
+            const __nv_bfloat16 grad = __float2bfloat16_rn(2.f * inv * acc);
+            if ((reinterpret_cast<uintptr_t>(dy) & 15) == 0) {
+                uint4 w = make_uint4((unsigned)__bfloat16_as_ushort(grad), 0u, 0u, 0u);
 #pragma unroll
-            for (int q = 0; q < 8; q++) {
-                d[q] = w;
-                w.x = 0u;
+                for (int q = 0; q < 8; q++) {
+                    reinterpret_cast<uint4 *>(d)[q] = w;
+                    w.x = 0u;
+                }
+            } else {
+                d[0] = grad;
+#pragma unroll 4
+                for (int c = 1; c < kC; c++) d[c] = __float2bfloat16_rn(0.f);
             }
         }
     }
