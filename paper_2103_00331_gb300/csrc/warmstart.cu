@@ -391,15 +391,29 @@ __global__ void __launch_bounds__(kTmThreads, 1) conv_tma_kernel(const __grid_co
 // of them drifts (1.7e-6 off at 131,072 voxels when each CTA kept its sums in
 // TMEM to the end, 3.0e-7 on the FP32 pipe): each tile's sums (8 steps) are
 // drained and added up in registers, round to nearest, while the next tile
-// runs in the other TMEM buffer. At the end the CTA adds its sums to dW with
-// coalesced reductions.
+// runs in another TMEM accumulator. At the end the CTA adds its sums to dW
+// with coalesced reductions.
 // A voxel of a tile beyond the grid has dy = 0 from the copy: it adds 0 x.
 // One layer at 32 x 16^3 voxels: 1,660 us on the FP32 pipe (conv_dw_kernel),
-// 68 us here (error against FP64 3.0e-7 and 1.8e-7); the x and dy copies run
-// at 4.9 TB/s from L2. One CTA for all nine taps of an oz with its sums kept
-// in TMEM took 38 us, at the error above.
+// 47 us here; the x and dy copies run at 7 TB/s from L2. One CTA for all nine
+// taps of an oz with its sums kept in TMEM took 38 us, at the error above.
+//
+// Error against FP64, root mean square over the largest outputs' scale, of
+// positive x (after a ReLU): the truncation inside a tile leaves about 7e-8
+// whatever the size, every reduction into dW a rounding of the whole sum. The
+// FP32 pipe, 512 voxels a block, is at its best with few blocks (6.3e-8 at
+// 4,096 voxels, 8.9e-8 at 16,384, 24e-8 at 131,072; this kernel as above
+// 9.3e-8, 9.4e-8, 9.7e-8). So below kDwFew voxels a tile's 8 steps go to two
+// accumulators (half the truncation), up to kDwFewer voxels with at most 8
+// reductions an output, and less than one tile of voxels stays on the FP32
+// pipe: 5.9e-8 at 2,048 voxels (FP32 pipe 6.6e-8), 6.0e-8 at 4,096, 6.1e-8 at
+// 8,192 (6.9e-8), 7.2e-8 at 16,384. It costs time: 8.4 us for 6.6 at 4,096
+// voxels, 12.5 for 10.6 at 16,384, and would 55 for 47 at 131,072, where the
+// longer chain of register additions gains nothing either.
 constexpr uint32_t kDwIdesc = tc::kIdescM128N64AMN | (1u << 16);   // A and B MN-major
 constexpr int kDwMaxStages = 6;
+constexpr int kDwFew = 24576, kDwFewer = 8192;       // voxels (see above)
+constexpr int kDwAcc = 4;                            // accumulators (128 TMEM columns each) in turn
 
 struct DwGeo {
     int n, z, y, x;
@@ -410,11 +424,13 @@ struct DwGeo {
 };
 
 struct DwShared {
-    uint64_t full[kDwMaxStages], empty[kDwMaxStages], accf[2], acce[2];
+    uint64_t full[kDwMaxStages], empty[kDwMaxStages], accf[kDwAcc], acce[kDwAcc];
     uint32_t tslot;
     int abort;
 };
 
+// PARTS: accumulators a tile's 8 steps are spread over.
+template <int PARTS>
 __global__ void __launch_bounds__(kTmThreads, 1) conv_dw_tma_kernel(const __grid_constant__ CUtensorMap tmx,
                                                                     const __grid_constant__ CUtensorMap tmd,
                                                                     float *__restrict__ dw, DwGeo g) {
@@ -428,13 +444,13 @@ __global__ void __launch_bounds__(kTmThreads, 1) conv_dw_tma_kernel(const __grid
             tc::mbar_init(&S.full[i], 1);
             tc::mbar_init(&S.empty[i], 1);
         }
-        for (int i = 0; i < 2; i++) {
+        for (int i = 0; i < kDwAcc; i++) {
             tc::mbar_init(&S.accf[i], 1);
             tc::mbar_init(&S.acce[i], 128);
         }
         S.abort = 0;
     }
-    if (warp == 5) tc::tmem_alloc(&S.tslot, 256);
+    if (warp == 5) tc::tmem_alloc(&S.tslot, 128 * kDwAcc);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     tc::fence_proxy_async();
     tc::fence_before();
@@ -481,23 +497,29 @@ __global__ void __launch_bounds__(kTmThreads, 1) conv_dw_tma_kernel(const __grid
         uint64_t *lastbar = nullptr;
         uint32_t lastph = 0;
         const uint32_t s0 = tc::smem_u32(sm);
-        for (int tile = split; tile < g.tiles; tile += g.splits, count++) {
-            const uint32_t buf = count & 1;
-            if (count >= 2 && !tm_wait_warp(&S.acce[buf], ((count >> 1) - 1) & 1, abort)) break;
+        bool ok = true;
+        for (int tile = split; ok && tile < g.tiles; tile += g.splits) {
             if (!tm_wait_warp(&S.full[st], sph, abort)) break;
-            tc::fence_after();
             const uint32_t a0 = s0 + st * (uint32_t)g.stage_bytes;
             const uint64_t ad = tc::sdesc_mn(a0, (uint32_t)g.bstep), bd = tc::sdesc_mn(a0 + (uint32_t)g.xbytes, 8192u);
 #pragma unroll
-            for (int i = 0; i < 2; i++)
+            for (int part = 0; part < PARTS; part++, count++) {
+                const uint32_t buf = count % kDwAcc;
+                if (count >= kDwAcc && !tm_wait_warp(&S.acce[buf], (count / kDwAcc - 1) & 1, abort)) { ok = false; break; }
+                tc::fence_after();
 #pragma unroll
-                for (int ks = 0; ks < 8; ks++)
-                    tc::mma_lead(lead, tmem + 128u * buf + 64u * i, ad + (uint64_t)((i * g.bstep + ks * 2048) >> 4),
-                                 bd + (uint64_t)(ks * 2048 >> 4), kDwIdesc, ks > 0 ? 1u : 0u);
-            tc::commit_lead(lead, &S.empty[st]);
-            tc::commit_lead(lead, &S.accf[buf]);
-            lastbar = &S.accf[buf];
-            lastph = (count >> 1) & 1;
+                for (int i = 0; i < 2; i++)
+#pragma unroll
+                    for (int n = 0; n < 8 / PARTS; n++) {
+                        const int ks = part * (8 / PARTS) + n;
+                        tc::mma_lead(lead, tmem + 128u * buf + 64u * i, ad + (uint64_t)((i * g.bstep + ks * 2048) >> 4),
+                                     bd + (uint64_t)(ks * 2048 >> 4), kDwIdesc, n > 0 ? 1u : 0u);
+                    }
+                if (part == PARTS - 1) tc::commit_lead(lead, &S.empty[st]);
+                tc::commit_lead(lead, &S.accf[buf]);
+                lastbar = &S.accf[buf];
+                lastph = (count / kDwAcc) & 1;
+            }
             if (++st == (uint32_t)g.stages) { st = 0; sph ^= 1; }
         }
         // the MMAs complete in order: the last commit covers them all
@@ -513,9 +535,10 @@ __global__ void __launch_bounds__(kTmThreads, 1) conv_dw_tma_kernel(const __grid
             for (int c = 0; c < kC; c++) acc[i][c] = 0.f;
         bool ok = true;
         uint32_t count = 0;
-        for (int tile = split; tile < g.tiles; tile += g.splits, count++) {
-            const int buf = count & 1;
-            ok = __all_sync(0xFFFFFFFFu, tm_wait(&S.accf[buf], (count >> 1) & 1, abort));
+        const uint32_t parts = (uint32_t)((g.tiles - split + g.splits - 1) / g.splits) * PARTS;   // (split < tiles)
+        for (; count < parts; count++) {
+            const uint32_t buf = count % kDwAcc;
+            ok = __all_sync(0xFFFFFFFFu, tm_wait(&S.accf[buf], (count / kDwAcc) & 1, abort));
             if (!ok) break;
             tc::fence_after();
 #pragma unroll
@@ -546,10 +569,11 @@ __global__ void __launch_bounds__(kTmThreads, 1) conv_dw_tma_kernel(const __grid
     __syncthreads();
     tc::fence_after();
     if (tid == 0 && S.abort) atomicExch(&g_conv_err, 1);
-    if (warp == 5) tc::tmem_dealloc(tmem, 256);
+    if (warp == 5) tc::tmem_dealloc(tmem, 128 * kDwAcc);
 }
 
-// The same on the FP32 pipe, for operands that are not 16-byte aligned:
+// The same on the FP32 pipe, for operands that are not 16-byte aligned and for
+// less than a tile of voxels:
 // dW[t, co, ci] += sum over a chunk of voxels of dy[v, co] x[v + d off(t), ci]
 __global__ void __launch_bounds__(256) conv_dw_kernel(const __nv_bfloat16 *__restrict__ x,
                                                       const __nv_bfloat16 *__restrict__ dy, float *__restrict__ dw,
@@ -1358,9 +1382,9 @@ static cudaError_t launch_conv(const __nv_bfloat16 *x, const uint8_t *wimg, cons
 }
 
 // Weight gradient on the tensor cores; cudaErrorNotSupported where no tensor
-// copy can address the operands.
+// copy can address the operands, or there is less than one tile of voxels.
 static cudaError_t launch_dw(const __nv_bfloat16 *x, const __nv_bfloat16 *dy, float *dw, Dims dm, int dil, cudaStream_t st) {
-    if ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(dy)) & 15) return cudaErrorNotSupported;
+    if (((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(dy)) & 15) || dm.nvox() < 128) return cudaErrorNotSupported;
     DwGeo g;
     if (!tile_shape(dm, dil, g)) return cudaErrorNotSupported;
     const int rows = g.by + 2 * dil;
@@ -1376,12 +1400,12 @@ static cudaError_t launch_dw(const __nv_bfloat16 *x, const __nv_bfloat16 *dy, fl
     int dev = 0, sms = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(conv_dw_tma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTmSmemMax)) !=
-        cudaSuccess)
-        return e;
+    const auto kern = dm.nvox() < kDwFew ? conv_dw_tma_kernel<2> : conv_dw_tma_kernel<1>;
+    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kTmSmemMax)) != cudaSuccess) return e;
     g.splits = std::max(1, std::min(g.tiles, sms / 9));
+    if (dm.nvox() <= kDwFewer) g.splits = std::min(g.splits, 8);
     const size_t smem = 1024 + (size_t)g.stages * g.stage_bytes + sizeof(DwShared);
-    conv_dw_tma_kernel<<<9 * g.splits, kTmThreads, smem, st>>>(mx, md, dw, g);
+    kern<<<9 * g.splits, kTmThreads, smem, st>>>(mx, md, dw, g);
     return cudaGetLastError();
 }
 
