@@ -159,8 +159,8 @@ __device__ __forceinline__ int slab_div(int e, float inv) { return __float2int_r
 // Largest |a - b| seen so far, as a double. Float values: the exact
 // difference of two floats is d + e with d = fl(a - b) and e the rounding
 // error (Knuth's two-sum), kept as that pair and widened once at the end, so
-// no state costs an FP64 instruction. NaN differences are skipped, as fmax
-// skips them.
+// no state costs an FP64 instruction (but for one whose difference is past the
+// largest float). NaN differences are skipped, as fmax skips them.
 template <typename T> struct SlabMax;
 template <> struct SlabMax<double> {
     double m = 0.0;
@@ -172,14 +172,19 @@ template <> struct SlabMax<double> {
 };
 template <> struct SlabMax<float> {
     float d = 0.f, e = 0.f;
+    double wide = 0.0;         // differences that overflow a float
     __device__ __forceinline__ void add(float a, float b) {
         float s = a - b;
         const float bb = s - a;
         float t = (a - (s - bb)) - (b + bb);
         if (s < 0.f) { s = -s; t = -t; }
+        if (isinf(s)) {
+            wide = fmax(wide, fabs((double)a - (double)b));
+            return;
+        }
         if (s > d || (s == d && t > e)) { d = s; e = t; }
     }
-    __device__ __forceinline__ double get() const { return isinf(d) ? (double)d : (double)d + (double)e; }
+    __device__ __forceinline__ double get() const { return fmax(wide, (double)d + (double)e); }
 };
 
 // A block's threads split over `nch` chains, and a chain's threads over a
