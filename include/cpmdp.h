@@ -206,8 +206,14 @@ void cpmdp_default_opts(cpmdp_solve_opts *opts);
  * factors, plus the obstacle and terminal correction, encoded per state;
  * dense -> the given factors. Copies rewards, codes and factors to device
  * `device` and allocates the solvers' scratch there (about 8 bytes per
- * state; dense adds 2 value tensors and the intermediates of its fused
- * sweeps, whole actions of them up to 1 GiB and at least one action).
+ * state; dense adds 17 bytes per state, its factors in both precisions as
+ * given and transposed, and, for models without fused sweeps, 24 bytes per
+ * state). The first FP32 or FP64 sweep of a dense model, also one inside a
+ * solve, takes the intermediates of its fused sweeps: a tensor of |S| values
+ * (rounded up to whole tiles) per rank term of as many actions as fit 1 GiB,
+ * at least one action, once or, for plans of three runs of modes and more,
+ * twice; FP32 and FP64 share them where they are as large. Without the memory
+ * for them it falls back on 24 bytes per state and one launch per mode.
  * FP32 solves of rows that are no multiple of 4 states add a padded copy of
  * the model when first called. device = -1 builds a host-only object
  * usable by cpmdp_factors_info and cpmdp_components only.

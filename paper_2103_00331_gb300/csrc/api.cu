@@ -124,7 +124,7 @@ static thread_local SolveHost t_solve_host;
 static void free_device(Factors &F) {
     // the arena holds d_code, d_R32, d_R64, d_cell, d_scratch, d_ctrl and,
     // for shapes the barrier-free solver takes, d_flow
-    void *ptrs[] = {F.d_arena, F.d_q, F.d_U32, F.d_U64, F.d_Ubf, F.d_lam32, F.d_lam64, F.d_dense_work,
+    void *ptrs[] = {F.d_arena, F.d_q, F.d_U32, F.d_U64, F.d_Ubf, F.d_lam32, F.d_lam64, F.d_dense_work, F.d_dense_chain,
                     F.d_Vd, F.d_RB, F.d_T, F.d_EB, F.d_Vbase, F.d_tc_err, F.flow_in_arena ? nullptr : F.d_flow,
                     F.d_pi_work, F.d_dense_loop};
     for (void *p : ptrs)
@@ -149,7 +149,7 @@ static void free_device(Factors &F) {
     F.d_code = nullptr; F.d_R32 = nullptr; F.d_R64 = nullptr; F.d_cell = nullptr;
     F.d_scratch = nullptr; F.d_q = nullptr; F.d_ctrl = nullptr; F.d_U32 = nullptr;
     F.d_U64 = nullptr; F.d_Ubf = nullptr; F.d_lam32 = nullptr; F.d_lam64 = nullptr;
-    F.d_dense_work = nullptr; F.d_Vd = nullptr; F.d_RB = nullptr; F.d_T = nullptr;
+    F.d_dense_work = nullptr; F.d_dense_chain = nullptr; F.d_Vd = nullptr; F.d_RB = nullptr; F.d_T = nullptr;
     F.d_EB = nullptr; F.d_Vbase = nullptr; F.d_tc_err = nullptr; F.d_pi_work = nullptr;
     F.d_flow = nullptr; F.flow_in_arena = false;
 }

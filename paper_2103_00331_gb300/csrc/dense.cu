@@ -5,7 +5,7 @@
 //
 // SIMT path: the fused mode-product chains of dense_slab.cuh. Models that have
 // no plan there (a mode too large for one block's tile, or no memory for the
-// intermediates) run one tiled mode-product kernel per (action, rank, mode). The
+// intermediates or the transposed factors) run one tiled mode-product kernel per (action, rank, mode). The
 // mode-d product of X (viewed as L x N_d x Rt, Rt = prod of the later mode
 // sizes) with U is the batched matrix product Y[l, i, r] = sum_j U[i, j]
 // X[l, j, r]; columns c = (l, r) are tiled 64 at a time, rows i 64 at a
@@ -199,6 +199,12 @@ __global__ void __launch_bounds__(256) mode_product_kernel(const T *__restrict__
     }
 }
 
+// Chain ping-pong (2) and rank accumulator of the per-mode kernels: 3 x |S| doubles.
+static cpmdp_status mode_buffers(Factors &F) {
+    if (!F.d_dense_chain) CPMDP_CUDA(malloc_any_time(&F.d_dense_chain, 3 * (size_t)F.nstates * sizeof(double)));
+    return CPMDP_OK;
+}
+
 cpmdp_status dense_prepare(Factors &F) {
     const size_t nf = F.dense_factors.size();
     std::vector<float> u32(nf);
@@ -207,26 +213,34 @@ cpmdp_status dense_prepare(Factors &F) {
     CPMDP_CUDA(cudaMalloc(&F.d_U64, nf * sizeof(double)));
     CPMDP_CUDA(cudaMemcpy(F.d_U32, u32.data(), nf * sizeof(float), cudaMemcpyHostToDevice));
     CPMDP_CUDA(cudaMemcpy(F.d_U64, F.dense_factors.data(), nf * sizeof(double), cudaMemcpyHostToDevice));
-    const size_t S = (size_t)F.nstates;
-    // chain ping-pong (2), rank accumulator, running best, Q of the current
-    // action: 5 x |S| doubles; argmax |S| bytes
-    F.dense_work_bytes = 5 * S * sizeof(double) + S + 256;
-    CPMDP_CUDA(cudaMalloc(&F.d_dense_work, F.dense_work_bytes));
-    return slab_prepare(F);
+    // running best, Q of the current action: 2 x |S| doubles; argmax |S| bytes
+    CPMDP_CUDA(cudaMalloc(&F.d_dense_work, (size_t)F.nstates * (2 * sizeof(double) + 1)));
+    const cpmdp_status s = slab_prepare(F);
+    if (s != CPMDP_OK) return s;
+    return slab_plan(F, sizeof(float)) && slab_plan(F, sizeof(double)) ? CPMDP_OK : mode_buffers(F);
+}
+
+// The fused chains' intermediates are up to 1 GiB a buffer, so they wait for a
+// sweep that uses them (a model that runs BF16x3 sweeps alone never does).
+cpmdp_status dense_ready(const Factors &F, size_t elem) {
+    slab_workspace(F, elem);
+    return slab_plan(F, elem) ? CPMDP_OK : mode_buffers(const_cast<Factors &>(F));
 }
 
 template <typename T>
 static cpmdp_status dense_sweep(const Factors &F, const T *Vin, T *Vout, uint8_t *pi, int mode,
                                 double margin, unsigned long long *res, unsigned *chg, cudaStream_t st,
                                 const int *stop = nullptr) {
+    const cpmdp_status ready = dense_ready(F, sizeof(T));
+    if (ready != CPMDP_OK) return ready;
     if (slab_plan(F, sizeof(T))) {
         CPMDP_CUDA(slab_sweep<T>(F, Vin, Vout, pi, mode, (T)margin, res, chg, stop, st));
         return CPMDP_OK;
     }
     const size_t S = (size_t)F.nstates;
-    T *work = (T *)F.d_dense_work;
-    T *buf0 = work, *buf1 = work + S, *E = work + 2 * S, *best = work + 3 * S, *qold = work + 4 * S;
-    uint8_t *arg = (uint8_t *)(work + 5 * S);
+    T *const chain = (T *)F.d_dense_chain, *const work = (T *)F.d_dense_work;
+    T *buf0 = chain, *buf1 = chain + S, *E = chain + 2 * S, *best = work, *qold = work + S;
+    uint8_t *arg = (uint8_t *)(work + 2 * S);
     const T *U = std::is_same<T, double>::value ? (const T *)F.d_U64 : (const T *)F.d_U32;
     const T *R = std::is_same<T, double>::value ? (const T *)F.d_R64 : (const T *)F.d_R32;
     const int D = F.ndim;
@@ -492,6 +506,8 @@ static cpmdp_status dense_solve_t(const Factors &F, bool pim, T *V, uint8_t *pi,
     // buffers the recorded graph uses must exist before the recording
     if (!M.d_dense_loop) CPMDP_CUDA(cudaMalloc(&M.d_dense_loop, kLoopCtlBytes));
     if (!M.d_tc_err) CPMDP_CUDA(cudaMalloc(&M.d_tc_err, sizeof(int)));
+    const cpmdp_status ready = dense_ready(F, sizeof(T));
+    if (ready != CPMDP_OK) return ready;
     const int prec = std::is_same<T, double>::value ? 1 : 0;
     const bool same = M.simt_graph && M.simt_graph_V == (void *)V && M.simt_graph_pi == (void *)pi &&
                       M.simt_graph_pim == (int)pim && M.simt_graph_prec == prec && M.simt_graph_tol == o.tol &&

@@ -4,6 +4,7 @@
 
 #include <algorithm>
 #include <new>
+#include <type_traits>
 #include <vector>
 
 #include "dense_slab.cuh"
@@ -181,9 +182,13 @@ static void make_plan(const Factors &F, SlabPlan &plan) {
     }
     if (off > (1LL << 28)) return;
     plan.ublock = off;
-    // Intermediates of whole actions per group of launches: all of them up to 1 GiB, at least one action.
-    const double per = (double)F.rank * (double)F.nstates * sizeof(T);
-    plan.actions = (int)std::max(1.0, std::min((double)F.nactions, std::floor((double)(1u << 30) / per)));
+    // Intermediates of whole actions per group of launches: all of them up to
+    // 1 GiB a buffer, at least one action.
+    auto groups = [&](long long chain) {
+        const double per = (double)F.rank * (double)chain * sizeof(T);
+        return (int)std::max(1.0, std::min((double)F.nactions, std::floor((double)(1u << 30) / per)));
+    };
+    plan.actions = groups(F.nstates);
     const int nch = plan.actions * F.rank;
     // cheapest cut of the dimensions into phases
     double cost[kMaxDim + 1];
@@ -216,8 +221,9 @@ static void make_plan(const Factors &F, SlabPlan &plan) {
         z.inv_wprev = 1.f / (float)y.w;
         plan.chain = y.L * ((y.Rt + y.w - 1) / y.w) * y.w * y.G;   // whole tiles
         plan.chain = (std::max<long long>(plan.chain, F.nstates) + 3) & ~3LL;
+        plan.actions = groups(plan.chain);
     }
-    plan.ws_bytes = n > 1 ? (size_t)(n > 2 ? 2 : 1) * (size_t)nch * (size_t)plan.chain * sizeof(T) : 0;
+    plan.ws_bytes = n > 1 ? (size_t)(n > 2 ? 2 : 1) * (size_t)plan.actions * F.rank * (size_t)plan.chain * sizeof(T) : 0;
 }
 
 template <typename T>
@@ -241,7 +247,8 @@ void slab_free(Factors &F) {
     cudaFree(F.slab->ut64);
     cudaFree(F.slab->lam32);
     cudaFree(F.slab->lam64);
-    cudaFree(F.slab->ws);
+    cudaFree(F.slab->ws32);
+    if (F.slab->ws64 != F.slab->ws32) cudaFree(F.slab->ws64);
     delete F.slab;
     F.slab = nullptr;
 }
@@ -271,32 +278,50 @@ cpmdp_status slab_prepare(Factors &F) {
     }
     g.sblock = so;
     g.dblock = dof;
-    // The workspace is an option: without the memory for it the plans are dropped.
-    size_t ws = 0;
-    if (s->plan32.nphase) ws = std::max(ws, s->plan32.ws_bytes);
-    if (s->plan64.nphase) ws = std::max(ws, s->plan64.ws_bytes);
-    if (ws && cudaMalloc(&s->ws, ws) != cudaSuccess) {
-        (void)cudaGetLastError();
-        s->ws = nullptr;
-        s->plan32.nphase = s->plan64.nphase = 0;
-        return CPMDP_OK;
-    }
+    // A plan is an option: without the memory for its factors it is dropped.
     const dim3 grid(16, (unsigned)nch);
-    if (s->plan32.nphase) {
-        CPMDP_CUDA(cudaMalloc(&s->ut32, nch * (size_t)dof * sizeof(float)));
-        CPMDP_CUDA(cudaMalloc(&s->lam32, nch * sizeof(float)));
-        slab_transpose_kernel<float><<<grid, 256>>>(F.d_U64, s->ut32, g);
-        CPMDP_CUDA(cudaGetLastError());
-        CPMDP_CUDA(cudaMemcpy(s->lam32, l32.data(), nch * sizeof(float), cudaMemcpyHostToDevice));
-    }
-    if (s->plan64.nphase) {
-        CPMDP_CUDA(cudaMalloc(&s->ut64, nch * (size_t)dof * sizeof(double)));
-        CPMDP_CUDA(cudaMalloc(&s->lam64, nch * sizeof(double)));
-        slab_transpose_kernel<double><<<grid, 256>>>(F.d_U64, s->ut64, g);
-        CPMDP_CUDA(cudaGetLastError());
-        CPMDP_CUDA(cudaMemcpy(s->lam64, F.lambda.data(), nch * sizeof(double), cudaMemcpyHostToDevice));
-    }
+    auto put = [&](SlabPlan &plan, auto *&ut, auto *&lam, const void *host) -> cudaError_t {
+        typedef typename std::remove_reference<decltype(*ut)>::type T;
+        if (!plan.nphase) return cudaSuccess;
+        if (cudaMalloc(&ut, nch * (size_t)dof * sizeof(T)) != cudaSuccess ||
+            cudaMalloc(&lam, nch * sizeof(T)) != cudaSuccess) {
+            (void)cudaGetLastError();
+            cudaFree(ut);
+            ut = nullptr;
+            plan.nphase = 0;
+            return cudaSuccess;
+        }
+        slab_transpose_kernel<T><<<grid, 256>>>(F.d_U64, ut, g);
+        const cudaError_t e = cudaGetLastError();
+        return e != cudaSuccess ? e : cudaMemcpy(lam, host, nch * sizeof(T), cudaMemcpyHostToDevice);
+    };
+    CPMDP_CUDA(put(s->plan32, s->ut32, s->lam32, l32.data()));
+    CPMDP_CUDA(put(s->plan64, s->ut64, s->lam64, F.lambda.data()));
     return CPMDP_OK;
+}
+
+cudaError_t malloc_any_time(void **p, size_t bytes) {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    const cudaError_t e = cudaMalloc(p, bytes);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    return e;
+}
+
+void slab_workspace(const Factors &F, size_t elem) {
+    if (!F.slab) return;
+    DenseSlab &s = *F.slab;
+    SlabPlan &plan = elem == 8 ? s.plan64 : s.plan32;
+    void *&ws = elem == 8 ? s.ws64 : s.ws32;
+    if (!plan.nphase || !plan.ws_bytes || ws) return;
+    void *const other = elem == 8 ? s.ws32 : s.ws64;
+    if (other && (elem == 8 ? s.plan32 : s.plan64).ws_bytes >= plan.ws_bytes) {
+        ws = other;
+    } else if (malloc_any_time(&ws, plan.ws_bytes) != cudaSuccess) {
+        (void)cudaGetLastError();
+        ws = nullptr;
+        plan.nphase = 0;
+    }
 }
 
 const SlabPlan *slab_plan(const Factors &F, size_t elem) {
@@ -335,9 +360,9 @@ cudaError_t slab_sweep(const Factors &F, const T *Vin, T *Vout, uint8_t *pi, int
     a.mode = mode;
     a.gamma = (T)F.gamma;
     a.margin = margin;
-    a.best = work + 3 * S;
-    a.qold = work + 4 * S;
-    a.arg = (uint8_t *)(work + 5 * S);
+    a.best = work;
+    a.qold = work + S;
+    a.arg = (uint8_t *)(work + 2 * S);
     a.R = f64 ? (const T *)F.d_R64 : (const T *)F.d_R32;
     a.Vin = Vin;
     a.Vout = Vout;
@@ -359,7 +384,7 @@ cudaError_t slab_sweep(const Factors &F, const T *Vin, T *Vout, uint8_t *pi, int
             a.X = X;
             a.xchain = i == 0 ? 0 : plan.chain;
             a.ytiled = i == plan.nphase - 2;
-            a.Y = last ? nullptr : (T *)s.ws + (i & 1) * part;
+            a.Y = last ? nullptr : (T *)(f64 ? s.ws64 : s.ws32) + (i & 1) * part;
             const SlabPhase &p = a.p;
             const long long nx = last ? (p.L + p.w - 1) / p.w : p.L * ((p.Rt + p.w - 1) / p.w);
             const dim3 grid((unsigned)nx, last ? 1u : (unsigned)((a.nchains + p.ch - 1) / p.ch));

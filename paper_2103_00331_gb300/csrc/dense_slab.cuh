@@ -97,14 +97,15 @@ struct SlabPlan {
     size_t ws_bytes = 0;       // intermediates of one group (one buffer; two with 3 phases or more)
 };
 
-// The factors of every chain, transposed and padded, and the two plans.
+// The factors of every chain, transposed and padded, the two plans, and the
+// workspace of each (one allocation where the first one taken serves both).
 struct DenseSlab {
     SlabPlan plan32, plan64;
     float *ut32 = nullptr;
     double *ut64 = nullptr;
     float *lam32 = nullptr;
     double *lam64 = nullptr;
-    void *ws = nullptr;
+    void *ws32 = nullptr, *ws64 = nullptr;
 };
 
 template <typename T>
@@ -782,9 +783,11 @@ __global__ void __maxnreg__(IB * CB == 64 ? 168 : 128) slab_kernel(const __grid_
     }
 }
 
-// Build the plans, the transposed factors and the workspace (model build).
-// A model without a plan keeps slab == nullptr or nphase == 0.
+// Build the plans and the transposed factors (model build). A model without a
+// plan, or without the memory for its factors, has nphase == 0.
 cpmdp_status slab_prepare(Factors &F);
+// The workspace of sweeps of `elem`-byte values; without the memory for it the plan is dropped.
+void slab_workspace(const Factors &F, size_t elem);
 void slab_free(Factors &F);
 const SlabPlan *slab_plan(const Factors &F, size_t elem);
 

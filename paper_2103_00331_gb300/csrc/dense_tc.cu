@@ -960,6 +960,8 @@ cpmdp_status dense_tc_solve(const Factors &F, float *V, uint8_t *pi, const Solve
     // buffers the recorded graph uses must exist before the recording
     if (!M.d_dense_loop) CPMDP_CUDA(cudaMalloc(&M.d_dense_loop, kLoopCtlBytes));
     if (!M.d_Vd) CPMDP_CUDA(cudaMalloc(&M.d_Vd, (size_t)F.nstates * sizeof(double)));
+    if ((s = dense_ready(F, sizeof(float))) != CPMDP_OK) return s;
+    if ((s = dense_ready(F, sizeof(double))) != CPMDP_OK) return s;
     const int halve = F.gamma > 0.0 && F.gamma < 1.0 ? (int)ceil(log(2.0) / log(1.0 / F.gamma)) : 1;
     const bool same = M.dense_graph && M.dense_graph_V == (void *)V && M.dense_graph_pi == (void *)pi &&
                       M.dense_graph_tol == o.tol && M.dense_graph_max_iter == o.max_iter &&
@@ -1280,6 +1282,7 @@ cpmdp_status dense_tc_policy_iteration(const Factors &F, float *V, uint8_t *pi, 
     // buffers the recorded graph uses must exist before the recording
     if (!M.d_pi_work) CPMDP_CUDA(cudaMalloc(&M.d_pi_work, (size_t)kS * (2 * sizeof(float) + 1)));
     if (!M.d_dense_loop) CPMDP_CUDA(cudaMalloc(&M.d_dense_loop, kLoopCtlBytes));
+    if ((s = dense_ready(F, sizeof(float))) != CPMDP_OK) return s;
     const bool same = M.dense_pi_graph && M.dense_pi_graph_V == (void *)V && M.dense_pi_graph_pi == (void *)pi &&
                       M.dense_pi_graph_eval_tol == o.eval_tol && M.dense_pi_graph_rounds == o.max_rounds &&
                       M.dense_pi_graph_eval_iter == o.max_eval_iter && M.dense_pi_graph_partial == o.partial_eval;

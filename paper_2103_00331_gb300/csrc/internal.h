@@ -102,8 +102,8 @@ struct Factors {
     void *d_Ubf = nullptr;             // bf16 hi/lo split of the factors (tensor-core path)
     float *d_lam32 = nullptr;
     double *d_lam64 = nullptr;
-    void *d_dense_work = nullptr;      // dense chain intermediates
-    size_t dense_work_bytes = 0;
+    void *d_dense_work = nullptr;      // dense: running best, Q of the current action, argmax
+    void *d_dense_chain = nullptr;     // dense without fused chains: chain ping-pong, rank accumulator
     double *d_Vd = nullptr;            // dense FP64 certify: the float values as doubles
     DenseSlab *slab = nullptr;  // fused mode-product chains: plans, factors, workspace (dense_slab.cuh)
     // dense tensor-core path (64^4), allocated on first BF16X3 use
@@ -206,7 +206,11 @@ cpmdp_status dense_backup(const Factors &F, cpmdp_precision prec, const void *Vi
 cpmdp_status dense_solve(const Factors &F, cpmdp_precision prec, bool policy_iteration, void *V,
                          uint8_t *pi, const SolveOpts &o, Ctrl *host_ctrl, cudaStream_t st);
 cpmdp_status dense_prepare(Factors &F);
+// Device memory that sweeps of `elem`-byte values work in; taken by the first one.
+cpmdp_status dense_ready(const Factors &F, size_t elem);
 void slab_free(Factors &F);
+// cudaMalloc that a stream capture under way does not forbid.
+cudaError_t malloc_any_time(void **p, size_t bytes);
 // dense_tc.cu
 bool dense_tc_supported(const Factors &F);
 cpmdp_status dense_tc_backup(const Factors &F, const float *Vin, float *Vout, uint8_t *pi, double *res,
