@@ -413,7 +413,7 @@ __global__ void __launch_bounds__(kTmThreads, 1) conv_tma_kernel(const __grid_co
 constexpr uint32_t kDwIdesc = tc::kIdescM128N64AMN | (1u << 16);   // A and B MN-major
 constexpr int kDwMaxStages = 6;
 constexpr int kDwFew = 24576, kDwFewer = 8192;       // voxels (see above)
-constexpr int kDwAcc = 4;                            // accumulators (128 TMEM columns each) in turn
+constexpr int kDwAccMax = 4;                         // accumulators (128 TMEM columns each) in turn: two tiles'
 
 struct DwGeo {
     int n, z, y, x;
@@ -424,16 +424,19 @@ struct DwGeo {
 };
 
 struct DwShared {
-    uint64_t full[kDwMaxStages], empty[kDwMaxStages], accf[kDwAcc], acce[kDwAcc];
+    uint64_t full[kDwMaxStages], empty[kDwMaxStages], accf[kDwAccMax], acce[kDwAccMax];
     uint32_t tslot;
     int abort;
 };
 
-// PARTS: accumulators a tile's 8 steps are spread over.
+// PARTS: accumulators a tile's 8 steps are spread over. (A wait that runs out
+// leaves its role's loops by goto: a flag in their conditions cost 4 %.)
 template <int PARTS>
 __global__ void __launch_bounds__(kTmThreads, 1) conv_dw_tma_kernel(const __grid_constant__ CUtensorMap tmx,
                                                                     const __grid_constant__ CUtensorMap tmd,
                                                                     float *__restrict__ dw, DwGeo g) {
+    constexpr int kDwAcc = 2 * PARTS;
+    static_assert(kDwAcc <= kDwAccMax, "TMEM columns");
     extern __shared__ uint8_t smem_raw[];
     uint8_t *sm = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     DwShared &S = *reinterpret_cast<DwShared *>(sm + (size_t)g.stages * g.stage_bytes);
@@ -497,15 +500,14 @@ __global__ void __launch_bounds__(kTmThreads, 1) conv_dw_tma_kernel(const __grid
         uint64_t *lastbar = nullptr;
         uint32_t lastph = 0;
         const uint32_t s0 = tc::smem_u32(sm);
-        bool ok = true;
-        for (int tile = split; ok && tile < g.tiles; tile += g.splits) {
-            if (!tm_wait_warp(&S.full[st], sph, abort)) break;
+        for (int tile = split; tile < g.tiles; tile += g.splits) {
             const uint32_t a0 = s0 + st * (uint32_t)g.stage_bytes;
             const uint64_t ad = tc::sdesc_mn(a0, (uint32_t)g.bstep), bd = tc::sdesc_mn(a0 + (uint32_t)g.xbytes, 8192u);
 #pragma unroll
             for (int part = 0; part < PARTS; part++, count++) {
                 const uint32_t buf = count % kDwAcc;
-                if (count >= kDwAcc && !tm_wait_warp(&S.acce[buf], (count / kDwAcc - 1) & 1, abort)) { ok = false; break; }
+                if (count >= kDwAcc && !tm_wait_warp(&S.acce[buf], (count / kDwAcc - 1) & 1, abort)) goto issued;
+                if (part == 0 && !tm_wait_warp(&S.full[st], sph, abort)) goto issued;
                 tc::fence_after();
 #pragma unroll
                 for (int i = 0; i < 2; i++)
@@ -522,6 +524,7 @@ __global__ void __launch_bounds__(kTmThreads, 1) conv_dw_tma_kernel(const __grid
             }
             if (++st == (uint32_t)g.stages) { st = 0; sph ^= 1; }
         }
+    issued:
         // the MMAs complete in order: the last commit covers them all
         if (lastbar) tc::mbar_wait(lastbar, lastph, kCvWaitCycles);
         __syncwarp();
@@ -535,26 +538,29 @@ __global__ void __launch_bounds__(kTmThreads, 1) conv_dw_tma_kernel(const __grid
             for (int c = 0; c < kC; c++) acc[i][c] = 0.f;
         bool ok = true;
         uint32_t count = 0;
-        const uint32_t parts = (uint32_t)((g.tiles - split + g.splits - 1) / g.splits) * PARTS;   // (split < tiles)
-        for (; count < parts; count++) {
-            const uint32_t buf = count % kDwAcc;
-            ok = __all_sync(0xFFFFFFFFu, tm_wait(&S.accf[buf], (count / kDwAcc) & 1, abort));
-            if (!ok) break;
-            tc::fence_after();
+        for (int tile = split; tile < g.tiles; tile += g.splits) {
 #pragma unroll
-            for (int i = 0; i < 2; i++) {
-                if (i == 1 && half == 0) continue;   // oy = 0 again (whole warps)
+            for (int part = 0; part < PARTS; part++, count++) {
+                const int buf = count % kDwAcc;
+                ok = __all_sync(0xFFFFFFFFu, tm_wait(&S.accf[buf], (count / kDwAcc) & 1, abort));
+                if (!ok) goto drained;
+                tc::fence_after();
 #pragma unroll
-                for (int h = 0; h < 2; h++) {
-                    float v[32];
-                    tc::tmem_ld32(t0 + 128u * buf + 64u * i + 32u * h, v);
+                for (int i = 0; i < 2; i++) {
+                    if (i == 1 && half == 0) continue;   // oy = 0 again (whole warps)
 #pragma unroll
-                    for (int c = 0; c < 32; c++) acc[i][32 * h + c] += v[c];
+                    for (int h = 0; h < 2; h++) {
+                        float v[32];
+                        tc::tmem_ld32(t0 + 128u * buf + 64u * i + 32u * h, v);
+#pragma unroll
+                        for (int c = 0; c < 32; c++) acc[i][32 * h + c] += v[c];
+                    }
                 }
+                tc::fence_before();
+                tc::mbar_arrive(&S.acce[buf]);
             }
-            tc::fence_before();
-            tc::mbar_arrive(&S.acce[buf]);
         }
+    drained:
         if (ok) {
 #pragma unroll
             for (int i = 0; i < 2; i++) {
