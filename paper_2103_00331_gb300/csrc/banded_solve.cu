@@ -71,8 +71,8 @@ __global__ void __launch_bounds__(256) solve_vi_kernel(BandArgs a, T *V, T *Wbuf
 // dimensions; FP64, whose own pipe is the bound: 25.5 us at 1000 x 1000, 28.1
 // with three blocks).
 template <typename T, int D, int VEC>
-__global__ void __launch_bounds__(256, pi_one_segment<T, D>() ? 3 : 1) solve_pi_kernel(BandArgs a, T *V, T *Wbuf, uint8_t *pi, SolveParams sp,
-                                                       Ctrl *ctrl) {
+__global__ void __launch_bounds__(256, pi_one_segment<T, D>() ? 3 : 1)
+    solve_pi_kernel(BandArgs a, T *V, T *Wbuf, uint8_t *pi, SolveParams sp, Ctrl *ctrl) {
     typedef T TA;
     __shared__ unsigned shm[64];
     __shared__ unsigned shu[32];
@@ -377,8 +377,9 @@ static cudaError_t solve_t(const Factors &F, bool pim, T *V, uint8_t *pi, const 
     // gets a quarter of the SM's FP64 rate, so more warps of fewer states are
     // faster (10 x 10: 1.13 us a sweep with two states a thread).
     if (small_ok && F.nstates / vec <= kSmallMaxItems && 2 * (size_t)F.nstates * sizeof(T) <= 48 * 1024) {
-        if (vec == 1 || (sizeof(T) == 8 && F.nstates <= kSmallMaxItems)) { CPMDP_DISPATCH_D(F.ndim, e = (launch_small<T, DD, 1>(F, pim, V, pi, sp, trace, st))); }
-        else { CPMDP_DISPATCH_D(F.ndim, e = (launch_small<T, DD, V2>(F, pim, V, pi, sp, trace, st))); }
+        if (vec == 1 || (sizeof(T) == 8 && F.nstates <= kSmallMaxItems)) {
+            CPMDP_DISPATCH_D(F.ndim, e = (launch_small<T, DD, 1>(F, pim, V, pi, sp, trace, st)));
+        } else { CPMDP_DISPATCH_D(F.ndim, e = (launch_small<T, DD, V2>(F, pim, V, pi, sp, trace, st))); }
         return e;
     }
     if (pim) {

@@ -320,16 +320,15 @@ cpmdp_status dense_backup(const Factors &F, cpmdp_precision prec, const void *Vi
     return dense_tc_backup(F, (const float *)Vin, (float *)Vout, pi, res, st);
 }
 
-// Value / policy iteration for dense models: each sweep is A*R*D launches
-// of milliseconds of work, so the loop runs on the host and reads the
-// residual (8 bytes) back once per sweep.
 // ---------------------------------------------------------------------------
-// The SIMT loops as one CUDA graph launch each (conditional nodes; the same
-// sweeps and stop rules as a host-driven loop, no residual read back per
-// sweep). Value iteration: WHILE { sweep V -> W, control, IF(second: sweep
-// W -> V, control) }, IF(odd count: copy W -> V), greedy policy. Policy
-// iteration: greedy start, WHILE(round) { start, WHILE(eval) { evaluation
-// sweeps as above }, IF(odd: copy), improvement sweep, round end }.
+// The FP32 and FP64 loops as one CUDA graph launch each (conditional nodes; the
+// same sweeps and stop rules as a host-driven loop, no residual read back per
+// sweep). Value iteration with fused chains: WHILE { kSimtUnroll sweeps V -> W,
+// W -> V in turn, each with its control }; without: WHILE { sweep V -> W,
+// control, IF(second: sweep W -> V, control) }; then IF(odd count: copy W ->
+// V), greedy policy. Policy iteration: greedy start, WHILE(round) { start,
+// WHILE(eval) { evaluation sweeps in twos as without fused chains }, IF(odd:
+// copy), improvement sweep, round end }.
 
 // After value-iteration sweep `step` (0: V -> W, 1: W -> V; 2, 3: the same with
 // no conditional second half).
@@ -357,8 +356,10 @@ __global__ void simt_vi_ctl_kernel(DensePiCtl *c, unsigned long long *res_slot, 
 // Sweeps per turn of value iteration's loop where the fused chains run: a turn
 // of a conditional node costs about 6 us on the device, more than a sweep of a
 // small model, so a turn holds several sweeps, and those after the stopping one
-// return at once (8^4, FP64: 23.5 us a sweep with two sweeps a turn and the
-// second one conditional).
+// return after their first tile (8^4, FP64: 18 us a sweep, 23.5 with two sweeps
+// a turn and the second one conditional). On a large model a skipped sweep's
+// two launches read |S| values each, once: 7 of them cost 48 x 50 x 52 x 46 in
+// FP32 less than a tenth of one of its 1.55 ms sweeps, once a solve.
 constexpr int kSimtUnroll = 8;
 
 template <typename T>

@@ -99,11 +99,11 @@ cpmdp_status pad_prepare(Factors &F, cudaMemPool_t pool, cudaStream_t st) {
     P->code_bytes = F.code_bytes;
     P->num_sms = F.num_sms;
     P->d_ctrl = F.d_ctrl;
-    const size_t S = (size_t)P->nstates, cb = (size_t)F.code_bytes;
+    const size_t S = (size_t)P->nstates;
     auto up = [](size_t n) { return (n + 255) & ~(size_t)255; };
     const bool flow = flow_shape_ok(*P);
     const size_t o_R32 = up(S * sizeof(double)), o_W = o_R32 + up(S * sizeof(float)), o_V = o_W + up(S * sizeof(float));
-    const size_t o_code = o_V + up(S * sizeof(float)), o_pi = o_code + up(S * cb), o_flow = o_pi + up(S);
+    const size_t o_code = o_V + up(S * sizeof(float)), o_pi = o_code + up(S), o_flow = o_pi + up(S);
     const size_t total = o_flow + (flow ? up(flow_bytes(*P)) : 0);
     cudaError_t e = cudaMallocFromPoolAsync(&P->d_arena, total, pool, st);
     if (e != cudaSuccess) {
@@ -121,15 +121,11 @@ cpmdp_status pad_prepare(Factors &F, cudaMemPool_t pool, cudaStream_t st) {
     P->d_code = arena + o_code;
     P->pad_pi = reinterpret_cast<uint8_t *>(arena + o_pi);
     const int grid = grid_of(F, g.total);
-    const uint32_t wall = (uint32_t)((1ull << (2 * F.ndim)) - 1) | (1u << (2 * F.ndim));   // an obstacle's code
+    const uint8_t wall = (uint8_t)((1u << (2 * F.ndim)) - 1 | 1u << (2 * F.ndim));   // an obstacle's code
     pad_rows_kernel<double><<<grid, 256, 0, st>>>(F.d_R64, P->d_R64, g, 0.0);
     pad_rows_kernel<float><<<grid, 256, 0, st>>>(F.d_R32, P->d_R32, g, 0.f);
-    if (cb == 1)
-        pad_rows_kernel<uint8_t><<<grid, 256, 0, st>>>((const uint8_t *)F.d_code, (uint8_t *)P->d_code, g, (uint8_t)wall);
-    else if (cb == 2)
-        pad_rows_kernel<uint16_t><<<grid, 256, 0, st>>>((const uint16_t *)F.d_code, (uint16_t *)P->d_code, g, (uint16_t)wall);
-    else
-        pad_rows_kernel<uint32_t><<<grid, 256, 0, st>>>((const uint32_t *)F.d_code, (uint32_t *)P->d_code, g, wall);
+    // codes of at most three dimensions (pad_wanted) are one byte
+    pad_rows_kernel<uint8_t><<<grid, 256, 0, st>>>((const uint8_t *)F.d_code, (uint8_t *)P->d_code, g, wall);
     e = cudaGetLastError();
     if (e == cudaSuccess && flow) {
         P->d_flow = arena + o_flow;

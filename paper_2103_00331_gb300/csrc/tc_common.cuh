@@ -73,7 +73,7 @@ __device__ __forceinline__ void mma(uint32_t d_tmem, uint64_t a, uint64_t b, uin
 // the whole warp runs. The instruction takes its operands from uniform
 // registers: where one thread alone runs the loop (inside `if (lane == 0)`),
 // every descriptor is worked out in ordinary registers and moved over, about
-// 125 cycles for an MMA that the tensor cores finish in 50.
+// 125 cycles for an MMA that the tensor cores finish in about 80.
 __device__ __forceinline__ void mma_lead(bool lead, uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc,
                                          uint32_t accumulate) {
     asm volatile(
