@@ -896,7 +896,8 @@ def hbm_sweep(cp, dev, stream, peak):
 def kernel_case(name, reps=3):
     """Run one kernel workload a few times and exit (for ncu captures):
     sweep512 / sweep320 = fused FP32 backup of a 512^3 / 320^3 GridWorld; dense64 / dense64f64 = one
-    FP32 / FP64 SIMT sweep of the 64^4 dense CP model; dense64tc = one BF16x3 tensor-core sweep of it;
+    FP32 / FP64 SIMT sweep of the 64^4 dense CP model; dense48 / dense48f64 = the same of a
+    48 x 50 x 52 x 46 model (4 actions, rank 4); dense64tc = one BF16x3 tensor-core sweep of the 64^4 one;
     solve64 / pi64 = fused
     FP32 value / policy iteration of the 64^3 instance (barrier-free solver);
     solve64b / pi64b = the same on the grid-barrier solver; ws512 = the warm-start network on
@@ -951,6 +952,21 @@ def kernel_case(name, reps=3):
             torch.cuda.synchronize()
             flops = 2.0 * 64 * 4 * dc.nstates * dc.nactions * dc.rank
             print(f"dense 64^4 FP64 SIMT sweep: {e0.elapsed_time(e1):.3f} ms, {flops / e0.elapsed_time(e1) / 1e9:.3f} TFLOP/s")
+            Va, Vb = Vb, Va
+    elif name in ("dense48", "dense48f64"):
+        dc = ci.dense_cp((48, 50, 52, 46), 4, 4, 0.95, seed=0)
+        f = cp.build_factors(dc, device=0)
+        prec, dt = (cp.F64, torch.float64) if name.endswith("f64") else (cp.F32, torch.float32)
+        Va = torch.as_tensor(ci.random_values(dc.shape, seed=2).reshape(-1)).to(dev, dt)
+        Vb = torch.empty_like(Va)
+        res = torch.zeros(1, dtype=torch.float64, device=dev)
+        for i in range(reps):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            cp.bellman_backup(f, prec, Va, Vb, None, res)
+            e1.record()
+            torch.cuda.synchronize()
+            print(f"dense 48 x 50 x 52 x 46 {str(dt)[6:]} sweep: {e0.elapsed_time(e1):.3f} ms")
             Va, Vb = Vb, Va
     elif name == "dense64":
         dc = ci.config_dense_4d(side=64, seed=0)
@@ -1057,7 +1073,7 @@ def main():
     ap.add_argument("--skip-dense", action="store_true")
     ap.add_argument("--skip-warmstart", action="store_true")
     ap.add_argument("--cpu-seconds", type=float, default=12.0)
-    ap.add_argument("--kernel-case", choices=["sweep512", "sweep320", "solve64", "pi64", "solve64b", "pi64b", "dense64", "dense64f64", "batch4096", "batchres1024",
+    ap.add_argument("--kernel-case", choices=["sweep512", "sweep320", "solve64", "pi64", "solve64b", "pi64b", "dense64", "dense64f64", "dense48", "dense48f64", "batch4096", "batchres1024",
                                               "dense64tc", "ws512", "batch1024", "batchcert"],
                     default=None,
                     help="run one kernel workload a few times (profiling) and exit")
