@@ -179,11 +179,10 @@ template <> struct SlabMax<float> {
         const float bb = s - a;
         float t = (a - (s - bb)) - (b + bb);
         if (s < 0.f) { s = -s; t = -t; }
-        if (isinf(s)) {
-            wide = fmax(wide, fabs((double)a - (double)b));
-            return;
+        if (s > d || (s == d && t > e)) {
+            if (isinf(s)) wide = fmax(wide, fabs((double)a - (double)b));
+            else { d = s; e = t; }
         }
-        if (s > d || (s == d && t > e)) { d = s; e = t; }
     }
     __device__ __forceinline__ double get() const { return fmax(wide, (double)d + (double)e); }
 };
