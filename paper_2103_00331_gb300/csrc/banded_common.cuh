@@ -508,8 +508,8 @@ struct Segment {
 };
 
 // Whether the policy sweeps keep one segment in flight per thread (solve_pi_kernel).
-template <typename T, int D>
-constexpr bool pi_one_segment() { return sizeof(T) == 4 && D == 3; }
+template <typename T, int D, int VEC>
+constexpr bool pi_one_segment() { return sizeof(T) == 4 && D == 3 && VEC == 4; }
 
 // All segments of one sweep, grid-stride, two segments in flight per thread.
 // With a grid of co-resident blocks, the states being worked on at any time
@@ -521,7 +521,7 @@ __device__ __forceinline__ TA sweep_all(const BandArgs &a, const T *V, T *W, uin
     const int nitems = a.nstates / VEC;
     const int step = gridDim.x * blockDim.x;
     TA res = 0;
-    constexpr bool kOne = MODE != M_VI && pi_one_segment<T, D>();
+    constexpr bool kOne = MODE != M_VI && pi_one_segment<T, D, VEC>();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nitems; i += kOne ? step : 2 * step) {
         Segment<T, TA, D, VEC> s0, s1;
         const bool two = !kOne && i + step < nitems;

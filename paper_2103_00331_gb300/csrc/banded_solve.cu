@@ -64,14 +64,20 @@ __global__ void __launch_bounds__(256) solve_vi_kernel(BandArgs a, T *V, T *Wbuf
     }
 }
 
-// FP32, three dimensions: one segment in flight a thread and three blocks an
-// SM (sweep_all); 145 registers for two segments left one block an SM, 8
-// warps: 60.1 us a sweep at 200 x 208 x 212, 34.7 us so (7.1 and 6.3 us at
-// 101 x 97 x 103). Two segments stay where they are as fast or faster (two
-// dimensions; FP64, whose own pipe is the bound: 25.5 us at 1000 x 1000, 28.1
-// with three blocks).
+// FP32 segments of 4 states in three dimensions: one segment in flight a thread
+// and three blocks an SM (sweep_all); 145 registers for two segments left one
+// block an SM, 8 warps: 60.1 us a sweep at 200 x 208 x 212, 34.7 us so (7.1 and
+// 6.3 us at 101 x 97 x 103). Two segments stay where they are as fast or faster.
+// There the compiler is told of one block (1: as many registers as it likes)
+// where its own choice has one an SM anyway or the FP64 pipe is the bound (40
+// rounds at 160^3 in FP64 22.8 ms, 24.0 with its own; 1000 x 1000 4.40 and 4.62),
+// and of none (0) elsewhere: 147 registers in place of 111 left one block of two
+// (FP32, 4000 x 4000: 11.2 and 7.2 ms), 72 in place of 47 two of five (one state
+// a thread, 10^7 + 1 states: 10.8 and 6.0 ms).
 template <typename T, int D, int VEC>
-__global__ void __launch_bounds__(256, pi_one_segment<T, D>() ? 3 : 1)
+constexpr int pi_blocks() { return pi_one_segment<T, D, VEC>() ? 3 : VEC > 1 && (sizeof(T) == 8 || D > 3) ? 1 : 0; }
+template <typename T, int D, int VEC>
+__global__ void __launch_bounds__(256, (pi_blocks<T, D, VEC>()))
     solve_pi_kernel(BandArgs a, T *V, T *Wbuf, uint8_t *pi, SolveParams sp, Ctrl *ctrl) {
     typedef T TA;
     __shared__ unsigned shm[64];
