@@ -635,7 +635,7 @@ static cpmdp_status run_solver(const cpmdp_factors *h, cpmdp_precision prec, boo
     bool have_ctrl = false;
     // FP32 solves of rows that are no multiple of 4 states run on a padded
     // copy of the grid (where there is memory for one)
-    bool padded = pad_wanted(F, prec, o);
+    bool padded = pad_wanted(F, prec, pi_mode, o);
     if (padded) {
         cudaMemPool_t pool;
         CPMDP_CUDA(arena_pool(F.device, &pool));
@@ -647,7 +647,9 @@ static cpmdp_status run_solver(const cpmdp_factors *h, cpmdp_precision prec, boo
     if (F.kind == CPMDP_GRIDWORLD) {
         if (padded) {
             CPMDP_CUDA(pad_in(F, (const float *)V, s));
-            st = banded_solve(A, prec, pi_mode, A.pad_V, A.pad_pi, o, s);
+            SolveOpts po = o;
+            if (pad_grid_barrier(A, pi_mode)) po.fused = 2;
+            st = banded_solve(A, prec, pi_mode, A.pad_V, A.pad_pi, po, s);
             if (st == CPMDP_OK) CPMDP_CUDA(pad_out(F, (float *)V, pi_mode ? pi : nullptr, s));
         } else if (!plain) {
             st = banded_solve(F, prec, pi_mode, V, pi, o, s);
@@ -675,7 +677,7 @@ static cpmdp_status run_solver(const cpmdp_factors *h, cpmdp_precision prec, boo
             // one FP64 backup into scratch: residual + policy of the returned V
             uint8_t *pout = pi_mode ? nullptr : pi;
             st = banded_backup(F, CPMDP_F64, V, F.d_scratch, pout, cert, s);
-        } else if (padded) {
+        } else if (padded && !pad_certify_rows(A)) {
             const bool want = !pi_mode && pi;
             st = banded_certify(A, A.pad_V, want ? A.pad_pi : nullptr, cert, s);
             if (st == CPMDP_OK && want) CPMDP_CUDA(pad_out(F, nullptr, pi, s));

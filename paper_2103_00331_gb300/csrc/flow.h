@@ -17,6 +17,8 @@ size_t flow_bytes(const Factors &F);
 // True when the shape alone lets the barrier-free solver run value or
 // policy iteration (the build then reserves its buffers with the factors).
 bool flow_shape_ok(const Factors &F);
+// Segments in a thread's column on this solve (0: the shape does not fit).
+int flow_column(const Factors &F, bool policy_iteration);
 size_t flow_counter_bytes();
 // One cooperative launch on `st` (F.d_flow allocated, tags above F.flow_base
 // never written before). Fills the control block like banded_solve.

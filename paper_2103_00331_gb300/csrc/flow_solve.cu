@@ -985,12 +985,14 @@ bool flow_eligible(const Factors &F, bool policy_iteration, const void *V, const
     return sweeps < (1ll << 31);
 }
 
-bool flow_shape_ok(const Factors &F) {
-    if (F.ndim < 1 || F.ndim > 3 || F.num_sms <= 0) return false;
-    if (F.shape[F.ndim - 1] % 4 != 0 || F.nstates % 4 != 0 || F.nstates >= (1ll << 30)) return false;
+int flow_column(const Factors &F, bool policy_iteration) {
+    if (F.ndim < 1 || F.ndim > 3 || F.num_sms <= 0) return 0;
+    if (F.shape[F.ndim - 1] % 4 != 0 || F.nstates % 4 != 0 || F.nstates >= (1ll << 30)) return 0;
     FlowShape s;
-    return flow_pick_any(F, s, false) || flow_pick_any(F, s, true);
+    return flow_pick_any(F, s, policy_iteration) ? s.zs : 0;
 }
+
+bool flow_shape_ok(const Factors &F) { return flow_column(F, false) || flow_column(F, true); }
 
 size_t flow_bytes(const Factors &F) {
     return (size_t)kSlots * kNC * kLineWords * sizeof(u64) + (size_t)kRing * F.nstates * sizeof(u64);

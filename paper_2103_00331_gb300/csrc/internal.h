@@ -193,7 +193,11 @@ cpmdp_status banded_plain_vi(const Factors &F, cpmdp_precision prec, void *V, ui
 // padded.cu
 // Whether an FP32 GridWorld solve runs on padded rows, and the padded copy
 // (device buffers from `pool`).
-bool pad_wanted(const Factors &F, cpmdp_precision prec, const SolveOpts &o);
+bool pad_wanted(const Factors &F, cpmdp_precision prec, bool policy_iteration, const SolveOpts &o);
+// Whether a solve on the padded copy P takes the grid-barrier solver whatever
+// else its shape allows, and whether its certificate takes the rows as they are.
+bool pad_grid_barrier(const Factors &P, bool policy_iteration);
+bool pad_certify_rows(const Factors &P);
 cpmdp_status pad_prepare(Factors &F, cudaMemPool_t pool, cudaStream_t st);
 void pad_free(Factors &F);
 // Values into the padded copy; values and / or policy (nullable) out of it.

@@ -13,6 +13,7 @@
 
 #include "banded_common.cuh"
 #include "flow.h"
+#include "march.h"
 
 namespace cpmdp {
 
@@ -51,7 +52,11 @@ static PadGeom geom_of(const Factors &F) {
     return {n, (n + 3) & ~3, (int)(F.nstates / n * ((n + 3) & ~3))};
 }
 
-bool pad_wanted(const Factors &F, cpmdp_precision prec, const SolveOpts &o) {
+// Padded copies of at least kMarchMinStates and less than this run their value
+// iteration and their certificate without the marching sweep (pad_grid_barrier).
+constexpr int64_t kPadMarchStates = 28ll << 20;
+
+bool pad_wanted(const Factors &F, cpmdp_precision prec, bool policy_iteration, const SolveOpts &o) {
     if (F.kind != CPMDP_GRIDWORLD || prec != CPMDP_F32 || o.fused != 1 || o.inject_stall) return false;
     const int64_t n = F.shape[F.ndim - 1], pitch = (n + 3) & ~3ll;
     // Up to 256 states one block solves the grid (30 us of 38 sweeps in all).
@@ -62,7 +67,33 @@ bool pad_wanted(const Factors &F, cpmdp_precision prec, const SolveOpts &o) {
     // 67 x 65 x 66 722 -> 406 us, at 101 x 97 x 103 (past the barrier-free
     // solver's size) 1,230 -> 925 us; policy iteration there 1,443 -> 1,407 us.
     if (n % 4 == 0 || F.ndim > 3 || F.nstates <= 256 || F.nstates / n * pitch >= (1ll << 30)) return false;
-    return pitch * 3 <= n * 4;
+    if (pitch * 3 > n * 4) return false;
+    // A solve limited to a few sweeps ends before they have paid for the copies:
+    // one sweep at 301 x 299 45 us as it is, 61 padded; 12 sweeps 69 and 69, 24
+    // sweeps 92 and 80; 55 x 56 x 57 78 and 84 at 12 sweeps, 91 and 90 at 16. From
+    // 101 x 97 x 103 on one sweep pays (93 and 88).
+    const int64_t eval = std::min(o.partial_eval, o.max_eval_iter);
+    const int64_t sweeps = !policy_iteration ? o.max_iter : o.partial_eval > 0 ? o.max_rounds * (eval + 1) : 1ll << 40;
+    return sweeps >= 12 || F.nstates >= 800000;
+}
+
+// Columns of four segments make the barrier-free policy iteration of
+// three-dimensional grids slower than the grid barrier (20 rounds at 75 x 73 x
+// 74: 349 and 301 us, 326 on the rows as they are; two dimensions 248 and 292 at
+// 751 x 749). Up to 28 million states the grid barrier's 16-byte sweeps are
+// faster than the marching sweep: 100 sweeps at 203 x 207 x 209 3,694 and 4,597
+// us (4,004 on the rows as they are), 259 x 255 x 257 6,778 and 8,374 (7,512),
+// 321 x 319 x 318 11,810 and 10,812 (13,805).
+bool pad_grid_barrier(const Factors &P, bool policy_iteration) {
+    if (P.ndim != 3) return false;
+    return policy_iteration ? flow_column(P, true) == 4 : P.nstates >= kMarchMinStates && P.nstates < kPadMarchStates;
+}
+
+// The same sizes take the FP64 certificate on the rows as they are: 224 us less
+// at 203 x 207 x 209, 368 at 259 x 255 x 257, 93 at 321 x 319 x 318; 94 more at
+// 361 x 359 x 357, and 104 more at 189 x 190 x 191, which does not march.
+bool pad_certify_rows(const Factors &P) {
+    return P.ndim == 3 && P.nstates >= kMarchMinStates && P.nstates < kPadMarchStates;
 }
 
 void pad_free(Factors &F) {
