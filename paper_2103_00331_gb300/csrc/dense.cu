@@ -4,8 +4,9 @@
 // Eq. 1's + R, x gamma and max over actions, and the residual.
 //
 // SIMT path: the fused mode-product chains of dense_slab.cuh. Models that have
-// no plan there (a mode too large for one block's tile, or no memory for the
-// intermediates or the transposed factors) run one tiled mode-product kernel per (action, rank, mode). The
+// no plan there (a mode too large for one block's tile, or so long that a
+// block's walk through it is slower, or no memory for the intermediates or the
+// transposed factors) run one tiled mode-product kernel per (action, rank, mode). The
 // mode-d product of X (viewed as L x N_d x Rt, Rt = prod of the later mode
 // sizes) with U is the batched matrix product Y[l, i, r] = sum_j U[i, j]
 // X[l, j, r]; columns c = (l, r) are tiled 64 at a time, rows i 64 at a

@@ -167,6 +167,45 @@ static PhaseCost plan_phase(const Factors &F, int d0, int d1, int nchains, const
     return best;
 }
 
+// Whether one launch per mode is faster than the plan. A block of a phase reads
+// every factor of the phase whole, which a single SM does at about 50 GB/s (FP32;
+// FP64: the SM's multiply-adds); a mode-product launch splits a long mode's rows
+// over many blocks, and takes 0.11 us per contraction step (FP64 1.07), up to
+// 1.75 times that where the factors outgrow the L2. So modes of more than 1,024
+// states lose where one wave of blocks walks few chains. Measured, fused / one
+// launch per mode, FP32: 1,500 states 223 / 172 us with one chain, 385 / 333 with
+// two, 2,209 / 3,471 with twelve; 2,000 states 613 / 435 with two; 2,500 x 4 780
+// / 563 with two; 1,500 x 32 316 / 365 with two. FP64: 2,000 states 4,706 / 4,238
+// with two, 1,500 states 2,614 / 3,194.
+template <typename T>
+static bool modes_faster(const Factors &F, const SlabPlan &plan) {
+    constexpr bool f64 = sizeof(T) == 8;
+    const double chains = (double)F.nactions * F.rank, sms = F.num_sms;
+    double fused = 0, modes = 0, bytes = 0;
+    bool longer = false;
+    for (int d = 0; d < F.ndim; d++) {
+        const double n = (double)F.shape[d];
+        longer |= n > 1024;
+        modes += chains * std::max(3.0, (f64 ? 1.07 : 0.11) * n);
+        bytes += chains * n * n * sizeof(T);
+    }
+    if (!longer) return false;
+    if (!f64) modes *= std::min(1.75, std::max(1.0, bytes / (64 << 20)));
+    for (int i = 0; i < plan.nphase; i++) {
+        const SlabPhase &p = plan.ph[i];
+        const bool last = i == plan.nphase - 1;
+        const double blocks = last ? std::ceil((double)p.L / p.w) : (double)p.L * p.ntile * std::ceil(chains / p.ch);
+        const double passes = (last ? std::ceil(chains / p.ch) : p.ch) * std::ceil(blocks / sms);
+        double factor = 0;
+        for (int q = 0; q < p.nmodes; q++) {
+            if (last && blocks > sms && p.m[q].N > 1024) return false;
+            factor += (double)p.m[q].N * p.m[q].N;
+        }
+        fused += f64 ? 5.9e-4 * factor * passes : last ? 50 + 7.8e-5 * factor * passes : 1.25e-4 * factor * passes;
+    }
+    return fused > modes;
+}
+
 template <typename T>
 static void make_plan(const Factors &F, SlabPlan &plan) {
     const int D = F.ndim;
@@ -224,6 +263,7 @@ static void make_plan(const Factors &F, SlabPlan &plan) {
         plan.actions = groups(plan.chain);
     }
     plan.ws_bytes = n > 1 ? (size_t)(n > 2 ? 2 : 1) * (size_t)plan.actions * F.rank * (size_t)plan.chain * sizeof(T) : 0;
+    if (modes_faster<T>(F, plan)) plan.nphase = 0;
 }
 
 template <typename T>
