@@ -137,7 +137,8 @@ typedef struct {
                                 grid-barrier solver); FP32 GridWorld solves of
                                 1 to 3 dimensions whose rows are a multiple of 4 states (other rows:
                                 on a copy with the rows padded to it, where that adds at most a
-                                third and the memory is there) and that fit
+                                third, the memory is there and the solve may take 12 sweeps or has
+                                800,000 states) and that fit
                                 one co-resident grid at one thread per column of 1, 2 or 4 segments of
                                 4 states run barrier-free (sweeps synchronised through sweep-tagged
                                 values, the stopping rule checked three sweeps late; same values and
